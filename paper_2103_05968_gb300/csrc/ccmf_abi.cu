@@ -42,8 +42,8 @@ void abw_params(int v, int& vw, int& tj) {
 }
 template <typename T> int lines_blocks_per_sm(int, int, size_t);
 template <typename T> int wlines_blocks_per_sm(int, int, size_t);
-template <typename T> int update_vec_blocks_per_sm();
-template <typename T> int update_vec_half_blocks_per_sm(int);
+template <typename T> int update_blocks_per_sm(int, bool);
+template <typename T> void launch_expand_state(const Ctx<T>&, cudaStream_t);
 template <typename T> int ab_blocks_per_sm(int, size_t);
 template <typename T> void launch_init(const Ctx<T>&, cudaStream_t);
 template <typename T> void launch_iteration(const Ctx<T>&, cudaStream_t);
@@ -71,10 +71,11 @@ constexpr size_t kSmemBudget = 96 * 1024;
 constexpr size_t kSmemMax = 200 * 1024;   // dynamic shared memory of one block, at most
 constexpr int kMaxTimedIters = 2048;
 // update-pass variant per precision, from measurements on GB300: register vectors in
-// ticket-ordered chunks. FP32 is bandwidth-bound: with half the voxels per thread and two
-// blocks per SM (variant 11) a 512^3 pass takes 2.37 ms against 2.41 ms (variant 0) and
-// 4.1 TB/s for the pipelines; at 128^3 x 3, 0.1525 against 0.1538 ms. FP64 is ALU-bound.
-constexpr int kDefaultUpdateVariantF32 = 11;
+// ticket-ordered chunks. FP32 waits for memory: half the voxels per thread and three blocks per SM
+// (variant 12, 80 registers, no spills) take 1.58 ms per 512^3 pass against 1.79 ms with two blocks (variant 11) and
+// 1.86 ms with one block of 16-byte vectors (variant 0); 0.236 / 0.266 / 0.274 ms at 256^3. FP64 is ALU-bound:
+// 0.751 ms per 128^3 pass with 16-byte vectors, 0.785 ms with one voxel per thread.
+constexpr int kDefaultUpdateVariantF32 = 12;
 constexpr int kDefaultUpdateVariantF64 = 0;
 // the captured loop runs the solves of a batch as up to this many independent graph
 // branches, so that one branch's FFT pass (on-chip work) overlaps another branch's
@@ -277,8 +278,6 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     long long gu = (pl->g.N + kThreads - 1) / kThreads;
     if (gu > 608) gu = 608;
     sh.grid_update = (int)gu;
-    sh.vec_resident = (f64 ? update_vec_blocks_per_sm<double>() : update_vec_blocks_per_sm<float>()) * sms;
-    sh.vec_resident_half = 0;
     // TMA-staged update: tiles of J z rows with J * N3 <= 512 (FP32) / 256 (FP64) voxels,
     // J a power of two dividing N2; two stages must fit the shared memory of a block
     const int tv_max = f64 ? 256 : 512;
@@ -309,8 +308,6 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
         // the vector update with half the voxels per thread (8-byte vectors in FP32), two blocks per
         // SM (11) or three (12)
         sh.upd_variant = variant;
-        sh.vec_resident_half = (f64 ? update_vec_half_blocks_per_sm<double>(variant)
-                                    : update_vec_half_blocks_per_sm<float>(variant)) * sms;
     }
     if (is_abw_variant(variant)) {
         // warp-independent stored-divergence update: an item is tj rows of one z segment of 32 VW
@@ -418,6 +415,15 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     if (sh.upd_variant == 0 && variant >= 1 && sh.tma_rows > 0) sh.upd_variant = 1;
     if (explicit_variant && sh.upd_variant != variant) return CCMF_ERR_UNSUPPORTED_SIZE;
     r.update_variant = sh.upd_variant;
+    {
+        const int kind = n3 % W != 0 ? kUpdStrided
+                         : sh.upd_variant == 11 ? kUpdHalf2
+                         : sh.upd_variant == 12 ? kUpdHalf3
+                                                : kUpdFull;
+        const int okind = n3 % W != 0 ? kUpdStrided : kUpdFull;
+        sh.upd_resident = (f64 ? update_blocks_per_sm<double>(kind, false) : update_blocks_per_sm<float>(kind, false)) * sms;
+        sh.out_resident = (f64 ? update_blocks_per_sm<double>(okind, true) : update_blocks_per_sm<float>(okind, true)) * sms;
+    }
     sh.grid_partials = std::max(sh.grid_update, sh.grid_tma);
     if (sh.upd_variant >= 2 && sh.upd_variant <= 7) sh.grid_partials = std::max(sh.grid_partials, sh.grid_pipe);
     if (is_abw_variant(sh.upd_variant))
@@ -425,11 +431,11 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
                                          (int)ceil_div((long long)sh.ab.nq * sh.ab.nr * sh.ab.npass, kAbwWarps));
     else if (is_ab_variant(sh.upd_variant))
         sh.grid_partials = std::max(sh.grid_partials, sh.ab.nq * sh.ab.nr);
-    // the vector update pass (variant 0 and every final evaluation) keeps one slot per chunk
-    sh.grid_partials = (int)std::max<long long>(sh.grid_partials, vec_update_chunks(pl->g.N, f64 ? 2 : 4));
-    if (sh.upd_variant == 11 || sh.upd_variant == 12)
-        sh.grid_partials = (int)std::max<long long>(sh.grid_partials,
-                                                    vec_update_chunks(pl->g.N, f64 ? 1 : 2));
+    // the register update pass and every final evaluation keep one slot per chunk, whatever the voxels per
+    // thread group (4, 2 in FP32; 2, 1 in FP64)
+    for (int w = f64 ? 1 : 2; w <= (f64 ? 2 : 4); w *= 2)
+        sh.grid_partials = (int)std::max<long long>(
+            sh.grid_partials, f64 ? vec_update_chunks<double>(pl->g.N, w) : vec_update_chunks<float>(pl->g.N, w));
     // y / x passes: one block per k_z plane when the plane fits its shared memory, a
     // cluster of C blocks (C divides n1 and n2) sharing the plane through distributed
     // shared memory, or the three strided passes
@@ -626,6 +632,12 @@ bool is_device_ptr(const void* ptr) {
 }
 
 template <typename T>
+void set_state_format(Ctx<T>* c, bool zs) {
+    c->use_zs = zs;
+    c->p.zs = zs ? 1 : 0;
+}
+
+template <typename T>
 Ctx<T> make_ctx(const ccmf_plan* pl, unsigned char* ws, const T* gamma, long long gstride, const LoopConfig& cfg) {
     Ctx<T> c;
     memset(&c, 0, sizeof(c));
@@ -661,6 +673,9 @@ Ctx<T> make_ctx(const ccmf_plan* pl, unsigned char* ws, const T* gamma, long lon
     // the stored-divergence schedule needs the vector loads of gamma (a per-solve pointer
     // table is aligned by the batch API's allocations of whole fields)
     c.use_ab = is_ab_variant(pl->sh.upd_variant) && c.vec_update;
+    // the register update variants of FP32 write the (z, s) state; the others read and write (e, v)
+    set_state_format(&c, sizeof(T) == 4 && (pl->sh.upd_variant == 0 || pl->sh.upd_variant == 11 ||
+                                            pl->sh.upd_variant == 12));
     return c;
 }
 
@@ -1212,11 +1227,22 @@ int ccmf_state_export(const ccmf_plan* plan, const void* workspace, void* e, voi
                         st) != cudaSuccess)
         return CCMF_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return CCMF_ERR_CUDA;
-    // the current copy of solve s is (iters & 1)
+    // the current copy of solve s is (iters & 1); a (z, s) state is expanded into the other copy, which the next
+    // update overwrites
     const size_t one = plan->esize * 6 * (size_t)plan->g.N;
     const size_t copy = one * plan->batch;
+    auto is_zs = [&](int s) { return plan->prec == CCMF_FP32_MIXED && sc[s].zs_iter == sc[s].iters; };
+    bool any_zs = false;
+    for (int s = 0; s < plan->batch; ++s) any_zs = any_zs || is_zs(s);
+    if (any_zs && (e || v)) {
+        LoopConfig cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        const Ctx<float> c = make_ctx<float>(plan, const_cast<unsigned char*>(ws), nullptr, 0, cfg);
+        launch_expand_state<float>(c, st);
+        if (cudaGetLastError() != cudaSuccess) return CCMF_ERR_CUDA;
+    }
     for (int s = 0; s < plan->batch; ++s) {
-        const size_t src = (size_t)(sc[s].iters & 1) * copy + (size_t)s * one;
+        const size_t src = (size_t)((sc[s].iters ^ (is_zs(s) ? 1 : 0)) & 1) * copy + (size_t)s * one;
         if (e && cudaMemcpyAsync((unsigned char*)e + (size_t)s * one, ws + plan->off_e + src, one, cudaMemcpyDefault,
                                  st) != cudaSuccess)
             return CCMF_ERR_CUDA;
@@ -1253,6 +1279,7 @@ int ccmf_state_import(const ccmf_plan* plan, void* workspace, const void* e, con
         sc[s].rho = rho[s];
         sc[s].iters = iters[s];
         sc[s].ab_iter = -1;   // stored divergences are recomputed from the imported state
+        sc[s].zs_iter = -1;   // an (e, v) state
     }
     if (cudaMemcpyAsync(ws + plan->off_sc, sc.data(), sizeof(SolveScalars) * plan->batch, cudaMemcpyHostToDevice,
                         st) != cudaSuccess)
@@ -1419,7 +1446,7 @@ int ccmf_plan_launch_info(const ccmf_plan* plan, int* out, int capacity, int* co
     const LaunchShape& sh = plan->sh;
     const int grid_upd = is_abw_variant(sh.upd_variant) ? (int)ceil_div((long long)sh.ab.nq * sh.ab.nr * sh.ab.npass, kAbwWarps)
                          : is_ab_variant(sh.upd_variant) ? sh.ab.nq * sh.ab.nr
-                         : (sh.upd_variant == 11 || sh.upd_variant == 12) ? sh.vec_resident_half / std::max(1, plan->batch)
+                         : (sh.upd_variant == 11 || sh.upd_variant == 12) ? sh.upd_resident / std::max(1, plan->batch)
                          : sh.upd_variant >= 2 ? sh.grid_pipe
                          : sh.upd_variant == 1 ? sh.grid_tma
                                                : sh.grid_update;
@@ -1542,10 +1569,10 @@ int batch_persist_capture(ccmf_batch* bt, const std::vector<Ctx<T>>& ctx, unsign
         G.rsym_y = c.rsym[1];
         G.sym_z = c.sym[2];
         G.div_l = make_fastdiv((unsigned)L);
-        G.inv_n = (T)(1.0 / (double)c.g.N);
+        G.inv_n = (T)(poisson_scale<T>() / (double)c.g.N);
         G.vec_div = c.vec_div ? 1 : 0;
         G.upd_w = (sizeof(T) == 4 && aligned && pl->n3 % 2 == 0) ? 2 : 1;
-        G.nchunks = vec_update_chunks(c.g.N, G.upd_w);
+        G.nchunks = persist_chunks(c.g.N, G.upd_w);
         const long long pairs = ceil_div((long long)pl->n1 * pl->n2, 2);
         G.tiles[0] = (int)ceil_div(pairs, P);
         G.tiles[1] = (int)ceil_div((long long)pl->n3h * pl->n1, L);
@@ -1672,6 +1699,7 @@ int batch_solve_impl(ccmf_batch* bt, const void* const* gammas, const double* xi
             return CCMF_ERR_CUDA;
         ctx[b] = make_ctx<T>(pl, wsb, nullptr, 0, cfg);
         ctx[b].p.gptrs = reinterpret_cast<const T* const*>(ws + bt->gp_off[b]);
+        if (bt->persistent) set_state_format(&ctx[b], false);   // k_batch_persist keeps (e, v)
     }
     for (int b = 0; b < nb; ++b) {
         ctx[b].vec_update = ctx[b].vec_div && aligned;
@@ -1897,7 +1925,7 @@ int ccmf_batch_create(int count, const int* shapes, int precision, ccmf_batch** 
         off = align_up(off + sizeof(void*) * bt->members[b].size());
     }
     // tables of the persistent launch (sized for either precision) and its chunk partial slots
-    // (one per chunk of kVecChunkGroups x kThreads voxels, the narrowest update vectors)
+    // (one per chunk of the update pass with the narrowest vectors)
     bt->pers_groups_off = off;
     off = align_up(off + sizeof(PersistGroup<double>) * keys.size());
     bt->pers_map_off = off;
@@ -1911,7 +1939,7 @@ int ccmf_batch_create(int count, const int* shapes, int precision, ccmf_batch** 
         size_t po = 0;
         for (ccmf_plan* pl : bt->plans) {
             bt->pers_part_b.push_back(po);
-            po = align_up(po + sizeof(double) * kNSum * (size_t)pl->batch * (size_t)vec_update_chunks(pl->g.N, 1));
+            po = align_up(po + sizeof(double) * kNSum * (size_t)pl->batch * (size_t)persist_chunks(pl->g.N, 1));
         }
         off = align_up(off + po);
     }
@@ -2112,8 +2140,8 @@ int adjoint_impl(ccmf_plan* pl, const T* gamma, long long gstride, const double*
     cfg.rho_sched = dsched;
     cfg.sched_len = K;
     Ctx<T> c = make_ctx<T>(pl, ws, gamma, gstride, cfg);
-    c.vec_update = false;   // the scalar update pass can also emit z
-    c.use_ab = false;
+        c.use_ab = false;
+    set_state_format(&c, false);   // checkpoints of (e, v)
     const size_t f6 = (size_t)6 * g.N * B;
     T* ckpt = reinterpret_cast<T*>(aws + L.ckpt);
     T* e_state = reinterpret_cast<T*>(ws + pl->off_e);
@@ -2349,8 +2377,8 @@ int adjoint_mixed_impl(ccmf_plan* pl, const float* gamma, long long gstride, con
 
     // FP64 forward replay with FP64 checkpoints of (e, v)
     Ctx<double> c64 = make_ctx<double>(p64, ws64, gam64, gstride64, cfg);
-    c64.vec_update = false;   // the scalar update pass can also emit z
-    c64.use_ab = false;
+        c64.use_ab = false;
+    set_state_format(&c64, false);
     const size_t f6 = (size_t)6 * N * B;
     double* ckpt = reinterpret_cast<double*>(aws + L.ckpt);
     double* e_state = reinterpret_cast<double*>(ws64 + p64->off_e);
@@ -2394,6 +2422,7 @@ int adjoint_mixed_impl(ccmf_plan* pl, const float* gamma, long long gstride, con
     // FP32 reverse sweep; the FP32 context supplies the M applications and the seed
     Ctx<float> c32 = make_ctx<float>(pl, ws, gamma, gstride, cfg);
     c32.use_ab = false;
+    set_state_format(&c32, false);
     launch_init<float>(c32, st);   // unit normals and gamma statistics of the FP32 workspace
     float* zbuf = reinterpret_cast<float*>(aws + L.z);
     unsigned* bits = reinterpret_cast<unsigned*>(aws + L.bits);

@@ -11,13 +11,13 @@
 //                       (the (div^- grad^+)^+ of Eq. 28), inverse FFT along x;
 //   4. k_fft_lines<2>   inverse FFT along y;
 //   5. k_irfft_z        complex-to-real inverse FFT along z -> phi;
-//   6. k_update<false>  xi^{k+1/2} = w - A(A* w - grad^+ phi - xi_bar) (= P_K(w),
+//   6. k_update         xi^{k+1/2} = w - A(A* w - grad^+ phi - xi_bar) (= P_K(w),
 //                       Eq. 28), over-relaxation, z = v + rho xi, node-wise
 //                       projection onto C_gamma (Eq. 19), e^{k+1}, v^{k+1}
 //                       (Eq. 30), block partial sums; the last block reduces
 //                       them in double and updates rho, the history and the stop
 //                       flag on the device (Eq. 31, BB / LTD scaling).
-// k_update<true> is the final evaluation: it writes the cut xi^{K+1/2} and the
+// (ccmf_update.cuh.) Its OUT instantiation is the final evaluation: it writes the cut xi^{K+1/2} and the
 // flow A* v^K instead of advancing the state.
 #pragma once
 
@@ -25,7 +25,7 @@
 
 #include <cooperative_groups.h>
 
-#include "ccmf_types.cuh"
+#include "ccmf_state.cuh"
 
 namespace ccmf {
 
@@ -63,22 +63,43 @@ __device__ __forceinline__ T warp_sum(T x) {
     return x;
 }
 
+// Sums of NQ <= 16 values over the lanes of a warp: lane l ends with the sum of value index(l), valid where
+// index(l) < NQ and l is even. Each step exchanges half of the values a lane still holds, so 16 values take 16
+// additions and shuffles instead of 5 each (in FP64 an addition of a warp occupies its SM for 16 cycles).
+template <typename T, int NQ>
+__device__ __forceinline__ T warp_sums(const T (&acc)[NQ], int lane, int& index) {
+    static_assert(NQ <= 16, "sixteen values");
+    T v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q] = q < NQ ? acc[q < NQ ? q : 0] : T(0);
+#pragma unroll
+    for (int m = 8; m >= 1; m /= 2) {
+        const int off = 2 * m;
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int q = 0; q < m; ++q) {
+            const T send = up ? v[q] : v[q + m], keep = up ? v[q + m] : v[q];
+            v[q] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+    index = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
 // Block reduction of NQ per-thread values (T) into one double each, written to
 // partial[b * NQ + q] (fixed order: warp shuffles, then the warps in turn).
 template <typename T, int NQ, int NT = kThreads>
 __device__ void block_store_partial(const T (&acc)[NQ], double* __restrict__ partial, long long b) {
-    __shared__ double red[NT / 32][NQ];
+    __shared__ T red[NT / 32][NQ];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        T s = warp_sum(acc[q]);
-        if (lane == 0) red[wid][q] = (double)s;
-    }
+    int q;
+    const T s = warp_sums<T, NQ>(acc, lane, q);
+    if ((lane & 1) == 0 && q < NQ) red[wid][q] = s;
     __syncthreads();
     if (threadIdx.x < NQ) {
-        double s = 0.0;
-        for (int w = 0; w < NT / 32; ++w) s += red[w][threadIdx.x];
-        partial[b * NQ + threadIdx.x] = s;
+        double t = 0.0;
+        for (int w = 0; w < NT / 32; ++w) t += (double)red[w][threadIdx.x];
+        partial[b * NQ + threadIdx.x] = t;
     }
 }
 
@@ -105,25 +126,29 @@ __device__ bool block_partials(T (&acc)[NQ], double* __restrict__ partial, unsig
     return block_ticket<NT>(counter, nblocks);
 }
 
-// Deterministic double reduction of nblocks x NQ partials by one block.
+// Deterministic double reduction of nblocks x NQ partials by one block; the result is complete in thread 0.
 template <int NQ, int NT = kThreads>
 __device__ void reduce_partials(const double* __restrict__ partial, int nblocks, double (&out)[NQ]) {
     __shared__ double red[NT / 32][NQ];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double acc[NQ];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += NT) s += __ldcg(partial + (size_t)b * NQ + q);
-        s = warp_sum(s);
-        if (lane == 0) red[wid][q] = s;
+    for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
+    for (int b = threadIdx.x; b < nblocks; b += NT)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) acc[q] += __ldcg(partial + (size_t)b * NQ + q);
+    int q;
+    const double s = warp_sums<double, NQ>(acc, lane, q);
+    if ((lane & 1) == 0 && q < NQ) red[wid][q] = s;
+    __syncthreads();
+    if (threadIdx.x < NQ) {
+        double t = 0.0;
+        for (int w = 0; w < NT / 32; ++w) t += red[w][threadIdx.x];
+        red[0][threadIdx.x] = t;   // column q is this thread's alone
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        double s = 0.0;
-        for (int w = 0; w < NT / 32; ++w) s += red[w][q];
-        out[q] = s;
-    }
+    for (int i = 0; i < NQ; ++i) out[i] = red[0][i];
 }
 
 // ---------------------------------------------------------------------------
@@ -269,6 +294,8 @@ __global__ void __launch_bounds__(kThreads) k_init_stats(Geom g, Ptrs<T> p, Loop
             S.rho = cfg.rho_sched ? cfg.rho_sched[(size_t)s * cfg.sched_len] : rho0;
             S.iters = 0;
             S.ab_iter = -1;
+            S.zs_iter = p.zs ? 0 : -1;
+            S.rho_prev = 1.0;
         }
         S.status = status;
         S.converged = 0;
@@ -287,6 +314,8 @@ __global__ void __launch_bounds__(kThreads) k_init_state(Geom g, Ptrs<T> p) {
     const long long cur = (long long)(S.iters & 1) * p.sstride + (long long)s * 6 * g.N;
     T* e = p.e + cur;
     T* v = p.v + cur;
+    // (z, s) format: z = A xi_bar with s = 0 and rho_prev = 1 reads as e = A xi_bar, v = 0
+    const int nv = p.zs ? 1 : 6;
     const long long stride = (long long)gridDim.x * kThreads;
     for (long long lin = (long long)blockIdx.x * kThreads + threadIdx.x; lin < g.N; lin += stride) {
         e[0 * g.N + lin] = a0;
@@ -295,56 +324,8 @@ __global__ void __launch_bounds__(kThreads) k_init_state(Geom g, Ptrs<T> p) {
         e[3 * g.N + lin] = a0;
         e[4 * g.N + lin] = a1;
         e[5 * g.N + lin] = a2;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) v[c * g.N + lin] = T(0);
+        for (int c = 0; c < nv; ++c) v[c * g.N + lin] = T(0);
     }
-}
-
-// ---------------------------------------------------------------------------
-// 16-byte vectors of the field type (4 floats or 2 doubles).
-// ---------------------------------------------------------------------------
-template <typename T> struct Vec16;
-template <> struct Vec16<float> {
-    using type = float4;
-    static constexpr int W = 4;
-    __device__ __forceinline__ static void ld(const float* __restrict__ p, float (&o)[4]) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(p));
-        o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
-    }
-    __device__ __forceinline__ static void st(float* p, const float (&o)[4]) {
-        *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
-    }
-};
-template <> struct Vec16<double> {
-    using type = double2;
-    static constexpr int W = 2;
-    __device__ __forceinline__ static void ld(const double* __restrict__ p, double (&o)[2]) {
-        const double2 t = __ldg(reinterpret_cast<const double2*>(p));
-        o[0] = t.x; o[1] = t.y;
-    }
-    __device__ __forceinline__ static void st(double* p, const double (&o)[2]) {
-        *reinterpret_cast<double2*>(p) = make_double2(o[0], o[1]);
-    }
-};
-
-// Neighbour offsets of the row (i, j) of a solve: rows (i+1, j), (i-1, j), (i, j+1), (i, j-1).
-struct RowNb {
-    long long row, ip, im, jp, jm;  // element offsets of k = 0 of each row
-};
-
-__device__ __forceinline__ RowNb row_neighbours(const Geom& g, unsigned row) {
-    const unsigned i = fdiv(row, g.div_n2);
-    const int j = (int)(row - i * (unsigned)g.n2);
-    const int ip = ((int)i + 1 == g.n1) ? 0 : (int)i + 1, im = (i == 0) ? g.n1 - 1 : (int)i - 1;
-    const int jp = (j + 1 == g.n2) ? 0 : j + 1, jm = (j == 0) ? g.n2 - 1 : j - 1;
-    RowNb r;
-    const long long n3 = g.n3;
-    r.row = (long long)row * n3;
-    r.ip = ((long long)ip * g.n2 + j) * n3;
-    r.im = ((long long)im * g.n2 + j) * n3;
-    r.jp = ((long long)i * g.n2 + jp) * n3;
-    r.jm = ((long long)i * g.n2 + jm) * n3;
-    return r;
 }
 
 // ---------------------------------------------------------------------------
@@ -352,6 +333,7 @@ __device__ __forceinline__ RowNb row_neighbours(const Geom& g, unsigned row) {
 // Line l = i * n2 + j of a solve; block b packs line pairs (2q, 2q+1) for
 // q in [b P, b P + P) as real and imaginary parts of one complex line.
 // d(p) = (1/sqrt2) sum_a [w1_a(p) - w1_a(p - e_a) + w2_a(p + e_a) - w2_a(p)].
+// FP64 leaves out the factor 1/sqrt2 (div_scale): see fold_h.
 // VEC: each thread reads W consecutive voxels of a line with 16-byte loads.
 // ---------------------------------------------------------------------------
 template <typename T, int P, bool VEC, bool AB = false>
@@ -366,15 +348,16 @@ __global__ void __launch_bounds__(kThreads) k_div_rfft_z(Geom g, Ptrs<T> p, Axis
     C* twl = reinterpret_cast<C*>(smem_raw);
     C* A = twl + g.n3;
     C* B = A + (size_t)g.n3 * stride;
-    for (int t = threadIdx.x; t < g.n3; t += kThreads) twl[t] = tw[t];
-    const T irho = T(1) / (T)p.sc[s].rho;
-    const T h = T(0.70710678118654752440084436210485);
+    __shared__ T recip[2];
+    if (threadIdx.x == 0) state_recip<T>(p.sc[s], recip);
+    __syncthreads();
+    const T irho = recip[0];
     const long long N = g.N;
-    const long long cur = (long long)(p.sc[s].iters & 1) * p.sstride + (long long)s * 6 * N;
-    const T* __restrict__ e = p.e + cur;
-    const T* __restrict__ v = p.v + cur;
+    const StateSrc<T> f = state_src<T>(p, p.sc[s], s, N, recip);
+    const bool zs = state_is_zs<T>(p.sc[s]);
     const long long L = (long long)g.n1 * g.n2;
     const long long l0 = (long long)blockIdx.x * 2 * P;
+    for (int t = threadIdx.x; t < g.n3; t += kThreads) twl[t] = tw[t];
     const int n3w = g.n3 / W;
     const int cnt = 2 * P * n3w;
     T* Ar = reinterpret_cast<T*>(A);
@@ -401,50 +384,19 @@ __global__ void __launch_bounds__(kThreads) k_div_rfft_z(Geom g, Ptrs<T> p, Axis
             const RowNb rn = row_neighbours(g, (unsigned)l);
             const int kp = (k0 + W == g.n3) ? 0 : k0 + W;      // first voxel after the group
             const int km = (k0 == 0) ? g.n3 - 1 : k0 - 1;        // last voxel before the group
-            if constexpr (VEC) {
-                T w[6][W], tmp_e[W], tmp_v[W];
-#pragma unroll
-                for (int c = 0; c < 6; ++c) {
-                    Vec16<T>::ld(e + c * N + rn.row + k0, tmp_e);
-                    Vec16<T>::ld(v + c * N + rn.row + k0, tmp_v);
-#pragma unroll
-                    for (int u = 0; u < W; ++u) w[c][u] = tmp_e[u] - tmp_v[u] * irho;
-                }
-                T xp[W], xm[W], yp[W], ym[W];
-                Vec16<T>::ld(e + 3 * N + rn.ip + k0, tmp_e);
-                Vec16<T>::ld(v + 3 * N + rn.ip + k0, tmp_v);
-#pragma unroll
-                for (int u = 0; u < W; ++u) xp[u] = tmp_e[u] - tmp_v[u] * irho;
-                Vec16<T>::ld(e + 0 * N + rn.im + k0, tmp_e);
-                Vec16<T>::ld(v + 0 * N + rn.im + k0, tmp_v);
-#pragma unroll
-                for (int u = 0; u < W; ++u) xm[u] = tmp_e[u] - tmp_v[u] * irho;
-                Vec16<T>::ld(e + 4 * N + rn.jp + k0, tmp_e);
-                Vec16<T>::ld(v + 4 * N + rn.jp + k0, tmp_v);
-#pragma unroll
-                for (int u = 0; u < W; ++u) yp[u] = tmp_e[u] - tmp_v[u] * irho;
-                Vec16<T>::ld(e + 1 * N + rn.jm + k0, tmp_e);
-                Vec16<T>::ld(v + 1 * N + rn.jm + k0, tmp_v);
-#pragma unroll
-                for (int u = 0; u < W; ++u) ym[u] = tmp_e[u] - tmp_v[u] * irho;
-                const T zp = __ldg(e + 5 * N + rn.row + kp) - __ldg(v + 5 * N + rn.row + kp) * irho;
-                const T zm = __ldg(e + 2 * N + rn.row + km) - __ldg(v + 2 * N + rn.row + km) * irho;
-#pragma unroll
-                for (int u = 0; u < W; ++u) {
-                    const T w2zp = (u + 1 < W) ? w[5][(u + 1) % W] : zp;
-                    const T w1zm = (u > 0) ? w[2][(u + W - 1) % W] : zm;
-                    const T sx = w[0][u] - xm[u] + xp[u] - w[3][u];
-                    const T sy = w[1][u] - ym[u] + yp[u] - w[4][u];
-                    const T sz = w[2][u] - w1zm + w2zp - w[5][u];
-                    d[u] = h * (sx + sy + sz);
-                }
+            auto div = [&](auto fmt) {
+                if constexpr (VEC)
+                    div_group<T, decltype(fmt)::value>(f, rn, k0, kp, km, d);
+                else
+                    d[0] = div_voxel<T, decltype(fmt)::value>(f, rn, k0, kp, km);
+            };
+            if constexpr (sizeof(T) == 4) {
+                if (zs)
+                    div(BoolC<true>{});
+                else
+                    div(BoolC<false>{});
             } else {
-                const long long p0 = rn.row + k0;
-                auto wc = [&](int c, long long off) { return e[c * N + off] - v[c * N + off] * irho; };
-                const T sx = wc(0, p0) - wc(0, rn.im + k0) + wc(3, rn.ip + k0) - wc(3, p0);
-                const T sy = wc(1, p0) - wc(1, rn.jm + k0) + wc(4, rn.jp + k0) - wc(4, p0);
-                const T sz = wc(2, p0) - wc(2, rn.row + km) + wc(5, rn.row + kp) - wc(5, p0);
-                d[0] = h * (sx + sy + sz);
+                div(BoolC<false>{});
             }
         }
 #pragma unroll
@@ -468,6 +420,14 @@ __global__ void __launch_bounds__(kThreads) k_div_rfft_z(Geom g, Ptrs<T> p, Axis
         if (lb < L) dst[1] = cmake<C>(T(0.5) * D.y, T(-0.5) * D.x);
     }
 }
+
+// -inv_n / lambda of the Poisson solve: the fast division in FP32 (relative error
+// 2 ulp, far below the FP32 field noise); in FP64 a Newton reciprocal.
+__device__ __forceinline__ float poisson_gain(float inv_n, float lam) { return __fdividef(-inv_n, lam); }
+__device__ __forceinline__ double poisson_gain(double inv_n, double lam) { return -inv_n * rcp_newton(lam); }
+// The same in the passes that divide exactly in FP32.
+__device__ __forceinline__ float poisson_gain_div(float inv_n, float lam) { return -inv_n / lam; }
+__device__ __forceinline__ double poisson_gain_div(double inv_n, double lam) { return poisson_gain(inv_n, lam); }
 
 // ---------------------------------------------------------------------------
 // Passes 2-4 for planes too large for one block: FFTs along y and x of the half
@@ -568,7 +528,7 @@ __global__ void __launch_bounds__(kThreads) k_fft_lines(Geom g, Ptrs<T> p, AxisP
             const T lam23 = valid ? rsym2[k2] + sym3[kz] : T(0);
             for (int m = m0; m < n; m += mstep) {
                 const T lam = rsym1[m] + lam23;
-                const T gk = (valid && lam > T(0)) ? -inv_n / lam : T(0);
+                const T gk = (valid && lam > T(0)) ? poisson_gain_div(inv_n, lam) : T(0);
                 const C z = b[m * stride + cl];
                 b[m * stride + cl] = cmake<C>(z.x * gk, -z.y * gk);
             }
@@ -627,11 +587,6 @@ constexpr int wlines_min_blocks() {
 
 template <int MODE, int N>
 __host__ __device__ constexpr int wlines_stride() { return N + N / 16 + (MODE == 1 ? 2 : 0); }
-
-// -inv_n / lambda of the Poisson solve: the fast division in FP32 (relative error
-// 2 ulp, far below the FP32 field noise), IEEE division in FP64.
-__device__ __forceinline__ float poisson_gain(float inv_n, float lam) { return __fdividef(-inv_n, lam); }
-__device__ __forceinline__ double poisson_gain(double inv_n, double lam) { return -inv_n / lam; }
 
 template <typename T, int MODE, int N>
 __global__ void __launch_bounds__(kThreads, wlines_min_blocks<T, MODE, N>())
@@ -814,7 +769,7 @@ __global__ void __launch_bounds__(plane_threads<T>(), 1) k_fft_plane(Geom g, Ptr
         const int i = (int)fdiv((unsigned)idx, g.div_n2);
         const int j = idx - i * n2;
         const T lam = rsym1[i] + rsym2[j] + l3;
-        const T gk = (lam > T(0)) ? -inv_n / lam : T(0);
+        const T gk = (lam > T(0)) ? poisson_gain_div(inv_n, lam) : T(0);
         const C z = tile[i * P2 + j];
         tile[i * P2 + j] = cmake<C>(z.x * gk, -z.y * gk);   // conj: the inverse runs as conj(DIT(conj))
     }
@@ -909,7 +864,7 @@ __global__ void __launch_bounds__(kPlaneClusterThreads, 1)
         const int cc = (int)fdiv((unsigned)e, g.div_n1);
         const int i = e - cc * n1;
         const T lam = rsym1[i] + rsym2[r * R2 + cc] + l3;
-        const T gk = (lam > T(0)) ? -inv_n / lam : T(0);
+        const T gk = (lam > T(0)) ? poisson_gain_div(inv_n, lam) : T(0);
         const C z = buf[cc * Q + i];
         buf[cc * Q + i] = cmake<C>(z.x * gk, -z.y * gk);   // conj: the inverse runs as conj(DIT(conj))
     }
@@ -974,14 +929,14 @@ __global__ void __launch_bounds__(kThreads, wz_min_blocks<T, N>())
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* twl = reinterpret_cast<C*>(smem_raw);
     C* lines = twl + N;
+    __shared__ T recip[2];
+    if (threadIdx.x == 0) state_recip<T>(p.sc[s], recip);
     warp_tw_fill<C, N>(twl, tw);
     __syncthreads();   // the twiddle table is filled by all threads of the block, then read by every warp
-    const T irho = T(1) / (T)p.sc[s].rho;
-    const T h = T(0.70710678118654752440084436210485);
+    const T irho = recip[0];
     const long long Nv = g.N;
-    const long long cur = (long long)(p.sc[s].iters & 1) * p.sstride + (long long)s * 6 * Nv;
-    const T* __restrict__ e = p.e + cur;
-    const T* __restrict__ v = p.v + cur;
+    const StateSrc<T> f = state_src<T>(p, p.sc[s], s, Nv, recip);
+    const bool zs = state_is_zs<T>(p.sc[s]);
     const long long L = (long long)g.n1 * g.n2;
     const long long l0 = (long long)blockIdx.x * RL;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1023,41 +978,13 @@ __global__ void __launch_bounds__(kThreads, wz_min_blocks<T, N>())
             } else if (valid) {
                 const int kp = (k0 + W == N) ? 0 : k0 + W;   // first voxel after the group
                 const int km = (k0 == 0) ? N - 1 : k0 - 1;   // last voxel before the group
-                T wv[6][W], te[W], tv[W];
-#pragma unroll
-                for (int c = 0; c < 6; ++c) {
-                    Vec16<T>::ld(e + c * Nv + rn.row + k0, te);
-                    Vec16<T>::ld(v + c * Nv + rn.row + k0, tv);
-#pragma unroll
-                    for (int u = 0; u < W; ++u) wv[c][u] = te[u] - tv[u] * irho;
-                }
-                T xp[W], xm[W], yp[W], ym[W];
-                Vec16<T>::ld(e + 3 * Nv + rn.ip + k0, te);
-                Vec16<T>::ld(v + 3 * Nv + rn.ip + k0, tv);
-#pragma unroll
-                for (int u = 0; u < W; ++u) xp[u] = te[u] - tv[u] * irho;
-                Vec16<T>::ld(e + 0 * Nv + rn.im + k0, te);
-                Vec16<T>::ld(v + 0 * Nv + rn.im + k0, tv);
-#pragma unroll
-                for (int u = 0; u < W; ++u) xm[u] = te[u] - tv[u] * irho;
-                Vec16<T>::ld(e + 4 * Nv + rn.jp + k0, te);
-                Vec16<T>::ld(v + 4 * Nv + rn.jp + k0, tv);
-#pragma unroll
-                for (int u = 0; u < W; ++u) yp[u] = te[u] - tv[u] * irho;
-                Vec16<T>::ld(e + 1 * Nv + rn.jm + k0, te);
-                Vec16<T>::ld(v + 1 * Nv + rn.jm + k0, tv);
-#pragma unroll
-                for (int u = 0; u < W; ++u) ym[u] = te[u] - tv[u] * irho;
-                const T zp = __ldg(e + 5 * Nv + rn.row + kp) - __ldg(v + 5 * Nv + rn.row + kp) * irho;
-                const T zm = __ldg(e + 2 * Nv + rn.row + km) - __ldg(v + 2 * Nv + rn.row + km) * irho;
-#pragma unroll
-                for (int u = 0; u < W; ++u) {
-                    const T w2zp = (u + 1 < W) ? wv[5][(u + 1) % W] : zp;
-                    const T w1zm = (u > 0) ? wv[2][(u + W - 1) % W] : zm;
-                    const T sx = wv[0][u] - xm[u] + xp[u] - wv[3][u];
-                    const T sy = wv[1][u] - ym[u] + yp[u] - wv[4][u];
-                    const T sz = wv[2][u] - w1zm + w2zp - wv[5][u];
-                    d[u] = h * (sx + sy + sz);
+                if constexpr (sizeof(T) == 4) {
+                    if (zs)
+                        div_group<T, true>(f, rn, k0, kp, km, d);
+                    else
+                        div_group<T, false>(f, rn, k0, kp, km, d);
+                } else {
+                    div_group<T, false>(f, rn, k0, kp, km, d);
                 }
             }
             // line 2w + q is the real (q = 0) or imaginary (q = 1) part of packed line w
@@ -1227,25 +1154,7 @@ template <typename T>
 struct StepConsts {
     T rho, irho, h, alpha, beta;
     T xi[3];
-};
-
-// Projection helpers. FP64 uses correctly rounded sqrt and division, as the
-// FP64 path is compared with the oracle at the 1e-10 level. FP32 uses the
-// hardware reciprocal square root (relative error ~1e-7, below FP32 field noise):
-// scale = gamma / |z| when |z| > gamma is gamma * rsqrt(|z|^2), compared in squares.
-template <typename T> struct Proj;
-template <> struct Proj<double> {
-    __device__ __forceinline__ static double scale(double nz2, double gm) {
-        const double nz = sqrt(nz2);
-        return (nz > gm) ? gm / nz : 1.0;
-    }
-    __device__ __forceinline__ static double norm(double x2) { return sqrt(x2); }
-};
-template <> struct Proj<float> {
-    __device__ __forceinline__ static float scale(float nz2, float gm) {
-        return (nz2 > gm * gm) ? gm * rsqrtf(nz2) : 1.0f;
-    }
-    __device__ __forceinline__ static float norm(float x2) { return x2 > 0.0f ? x2 * rsqrtf(x2) : 0.0f; }
+    T hxi[3];   // xi_bar / sqrt2
 };
 
 // Per-voxel work of the update pass. Inputs: the voxel's own state (ec, vc),
@@ -1266,12 +1175,17 @@ __device__ __forceinline__ void voxel_step(const StepConsts<T>& K, const T (&ec)
     for (int a = 0; a < 3; ++a) {
         const T w2p = e2p[a] - v2p[a] * K.irho;   // w2_a(p + e_a)
         const T w1m = e1m[a] - v1m[a] * K.irho;   // w1_a(p - e_a)
-        const T ua = K.h * (w[a] + w2p);          // (A* w)_a(p)
-        const T uam = K.h * (w1m + w[3 + a]);     // (A* w)_a(p - e_a)
-        const T ya = ua - (php[a] - ph0) - K.xi[a];
-        const T yam = uam - (ph0 - phm[a]) - K.xi[a];
-        xh[a] = w[a] - K.h * ya;
-        xh[3 + a] = w[3 + a] - K.h * yam;
+        if constexpr (fold_h<T>()) {
+            xh[a] = T(0.5) * (w[a] - w2p) + ((php[a] - ph0) + K.hxi[a]);
+            xh[3 + a] = T(0.5) * (w[3 + a] - w1m) + ((ph0 - phm[a]) + K.hxi[a]);
+        } else {
+            const T ua = K.h * (w[a] + w2p);          // (A* w)_a(p)
+            const T uam = K.h * (w1m + w[3 + a]);     // (A* w)_a(p - e_a)
+            const T ya = ua - (php[a] - ph0) - K.xi[a];
+            const T yam = uam - (ph0 - phm[a]) - K.xi[a];
+            xh[a] = w[a] - K.h * ya;
+            xh[3 + a] = w[3 + a] - K.h * yam;
+        }
     }
     T r2 = T(0), nx2 = T(0);
 #pragma unroll
@@ -1333,7 +1247,7 @@ __device__ __forceinline__ void voxel_step(const StepConsts<T>& K, const T (&ec)
 
 // Reduction epilogue of the update pass: block partials, then the last block of
 // the solve reduces them in double and runs the penalty / history / stop logic.
-template <typename T, bool OUT, int NT = kThreads, bool AB = false>
+template <typename T, bool OUT, int NT = kThreads, bool AB = false, bool ZS = false>
 __device__ void update_finish(const Geom& g, const Ptrs<T>& p, const LoopConfig& cfg, SolveScalars& S, int s,
                               double rho_d, const double* part, int nparts);
 
@@ -1348,38 +1262,61 @@ __device__ void update_epilogue(const Geom& g, const Ptrs<T>& p, const LoopConfi
 }
 
 // The last block of a solve's update pass: reduce the nparts partials in a fixed
-// order, then the penalty rule, the history row and the stop decision.
-template <typename T, bool OUT, int NT, bool AB>
+// order, then the penalty rule, the history row and the stop decision. All other blocks have finished, so this is a
+// serial stretch of every iteration: one warp spreads the divisions and square roots over its lanes.
+template <typename T, bool OUT, int NT, bool AB, bool ZS>
 __device__ void update_finish(const Geom& g, const Ptrs<T>& p, const LoopConfig& cfg, SolveScalars& S, int s,
                               double rho_d, const double* part, int nparts) {
+    const int lane = threadIdx.x;
+    const int kk = S.iters, call_start = S.call_start;
+    const double xi = lane < 3 ? S.xi[lane] : 0.0;
+    const double Nd = (double)g.N;
     double sums[kNSum];
     reduce_partials<kNSum, NT>(part, nparts, sums);
-    if (threadIdx.x != 0) return;
+    if (lane >= 32) return;
+    // lane q holds sum q
+    double mine = 0.0;
+#pragma unroll
+    for (int q = 0; q < kNSum; ++q)
+        if (lane == q) mine = sums[q];
+    const bool finite = __all_sync(0xffffffffu, isfinite(mine));
+    if (lane < kNSum) S.sums[lane] = mine;
+    const double mean = (lane == kSumRes ? fmax(mine, 0.0) : mine) / Nd;
+    double mv2 = 0.0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const double m = __shfl_sync(0xffffffffu, mean, kSumV + c);
+        mv2 += m * m;
+    }
+    const double res2 = __shfl_sync(0xffffffffu, mean, kSumRes), prim = __shfl_sync(0xffffffffu, mean, kSumPrimal);
+    // lane 0: the residual; lane 1: |<v>|
+    const double root = sqrt(lane == 0 ? res2 : mv2);
+    const double r = __shfl_sync(0xffffffffu, root, 0), mv = __shfl_sync(0xffffffffu, root, 1);
+    // <xi_bar, mean A* v^k>, the max-flow value of Eq. 12 at iteration k
+    const double hd = 0.70710678118654752440084436210485;
+    const int a3 = lane < 3 ? lane : 0;
+    const double v1 = __shfl_sync(0xffffffffu, mine, kSumV + a3), v2 = __shfl_sync(0xffffffffu, mine, kSumV + 3 + a3);
+    const double term = xi * hd * (v1 + v2) / Nd;
+    double dual = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) dual += __shfl_sync(0xffffffffu, term, a);
+    // quotients of the penalty rules: lane 0 the BB correlation, lane 1 the BB ratio, lane 2 rho / rho_step_max
+    const double sve = sums[kSumDvDe], see = sums[kSumDeDe], svv = sums[kSumDvDv];
+    const double den = lane == 0 ? sqrt(svv * see) : lane == 1 ? see : cfg.rho_step_max;
+    const double quot = (lane == 2 ? rho_d : sve) / den;
+    const double corr = __shfl_sync(0xffffffffu, quot, 0), ratio = __shfl_sync(0xffffffffu, quot, 1);
+    const double lo = __shfl_sync(0xffffffffu, quot, 2), hi = rho_d * cfg.rho_step_max;
+    if (lane != 0) return;
     S.counter = 0;
     S.chunk = 0;   // every block has left its work loop: the next launch starts from ticket 0
-    const double Nd = (double)g.N;
-    bool finite = true;
-    for (int q = 0; q < kNSum; ++q) {
-        S.sums[q] = sums[q];
-        finite = finite && isfinite(sums[q]);
-    }
-    const double r = sqrt(fmax(sums[kSumRes], 0.0) / Nd);
-    double mv2 = 0.0;
-    for (int c = 0; c < 6; ++c) mv2 += (sums[kSumV + c] / Nd) * (sums[kSumV + c] / Nd);
-    const double mv = sqrt(mv2);
-    const double prim = sums[kSumPrimal] / Nd;
     S.residual = r;
     S.mean_v = mv;
     S.primal = prim;
     if (OUT) {
-        const double hd = 0.70710678118654752440084436210485;
-        double dual = 0.0;
-        for (int a = 0; a < 3; ++a) dual += S.xi[a] * hd * (sums[kSumV + a] + sums[kSumV + 3 + a]) / Nd;
         S.dual = dual;
         if (!finite && S.status == 0) S.status = 5;
         return;
     }
-    const int kk = S.iters;
     if (cfg.hist_len > 0) {
         double* hrow = p.hist + ((size_t)s * kHistCap + (kk % cfg.hist_len)) * kHistFields;
         hrow[0] = (double)kk;
@@ -1387,19 +1324,13 @@ __device__ void update_finish(const Geom& g, const Ptrs<T>& p, const LoopConfig&
         hrow[2] = r;
         hrow[3] = mv;
         hrow[4] = prim;
-        const double hd = 0.70710678118654752440084436210485;
-        double dual = 0.0;   // <xi_bar, mean A* v^k>, the max-flow value of Eq. 12 at iteration k
-        for (int a = 0; a < 3; ++a) dual += S.xi[a] * hd * (sums[kSumV + a] + sums[kSumV + 3 + a]) / Nd;
         hrow[5] = dual;
     }
     double rho_new = rho_d;
-    const double lo = rho_d / cfg.rho_step_max, hi = rho_d * cfg.rho_step_max;
     if (cfg.rho_sched) {
         if (kk + 1 < cfg.sched_len) rho_new = cfg.rho_sched[(size_t)s * cfg.sched_len + kk + 1];
     } else if (cfg.rho_rule == 0) {
-        const double sve = sums[kSumDvDe], see = sums[kSumDeDe], svv = sums[kSumDvDv];
-        if (sve > 0.0 && see > 0.0 && svv > 0.0 && sve / sqrt(svv * see) > cfg.bb_corr_min)
-            rho_new = fmin(fmax(sve / see, lo), hi);
+        if (sve > 0.0 && see > 0.0 && svv > 0.0 && corr > cfg.bb_corr_min) rho_new = fmin(fmax(ratio, lo), hi);
     } else if (cfg.rho_rule == 2) {
         const double nv = sqrt(sums[kSumVV]), ne = sqrt(sums[kSumEE]);
         if (nv > 0.0 && ne > 0.0) rho_new = fmin(fmax(nv / ne, lo), hi);
@@ -1411,9 +1342,11 @@ __device__ void update_finish(const Geom& g, const Ptrs<T>& p, const LoopConfig&
         else if (sd > 10.0 * r)
             rho_new = lo;
     }
-    const int done = kk + 1 - S.call_start;
+    const int done = kk + 1 - call_start;
     S.iters = kk + 1;
     S.ab_iter = AB ? kk + 1 : -1;   // whether the pass also wrote the divergences of the new state
+    S.zs_iter = ZS ? kk + 1 : -1;   // the format of the new state
+    S.rho_prev = rho_d;
     bool stop = false;
     if (S.status != 0) {
         stop = true;   // a failure recorded during the pass (e.g. a bounded wait that gave up)
@@ -1445,256 +1378,15 @@ __device__ __forceinline__ StepConsts<T> step_consts(const SolveScalars& S, cons
     K.h = T(0.70710678118654752440084436210485);
     K.alpha = (T)(2.0 * (1.0 - cfg.delta));
     K.beta = (T)(1.0 - 2.0 * cfg.delta);
+    const double hd = 0.70710678118654752440084436210485;
     K.xi[0] = (T)S.xi[0];
     K.xi[1] = (T)S.xi[1];
     K.xi[2] = (T)S.xi[2];
+    K.hxi[0] = (T)(S.xi[0] * hd);
+    K.hxi[1] = (T)(S.xi[1] * hd);
+    K.hxi[2] = (T)(S.xi[2] * hd);
     return K;
 }
-
-// Scalar version (any N3, unaligned inputs, and the final evaluation pass).
-template <typename T, bool OUT>
-__global__ void __launch_bounds__(kThreads) k_update(Geom g, Ptrs<T> p, LoopConfig cfg) {
-    const int s = blockIdx.y + p.s0;
-    SolveScalars& S = p.sc[s];
-    if (!OUT && !S.active) return;
-    const long long N = g.N;
-    const double rho_d = S.rho;
-    const StepConsts<T> K = step_consts<T>(S, cfg);
-    // read the current copy of the state, write the other one (the stencil reads
-    // neighbours, so an in-place update would race)
-    const int par = S.iters & 1;
-    const T* __restrict__ e = p.e + (long long)par * p.sstride + (long long)s * 6 * N;
-    const T* __restrict__ v = p.v + (long long)par * p.sstride + (long long)s * 6 * N;
-    T* __restrict__ e_out = p.e + (long long)(1 - par) * p.sstride + (long long)s * 6 * N;
-    T* __restrict__ v_out = p.v + (long long)(1 - par) * p.sstride + (long long)s * 6 * N;
-    const T* __restrict__ phi = p.phi + (size_t)s * N;
-    const T* __restrict__ gam = gamma_of(p, s);
-    T acc[kNSum];
-#pragma unroll
-    for (int q = 0; q < kNSum; ++q) acc[q] = T(0);
-    const long long gstride = (long long)gridDim.x * kThreads;
-    for (long long lin = (long long)blockIdx.x * kThreads + threadIdx.x; lin < N; lin += gstride) {
-        const unsigned row = fdiv((unsigned)lin, g.div_n3);
-        const int k = (int)(lin - (long long)row * g.n3);
-        const RowNb rn = row_neighbours(g, row);
-        const int kp = (k + 1 == g.n3) ? 0 : k + 1, km = (k == 0) ? g.n3 - 1 : k - 1;
-        const long long nb_p[3] = {rn.ip + k, rn.jp + k, rn.row + kp};
-        const long long nb_m[3] = {rn.im + k, rn.jm + k, rn.row + km};
-        T ec[6], vc[6], php[3], phm[3], e2p[3], v2p[3], e1m[3], v1m[3];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            ec[c] = e[c * N + lin];
-            vc[c] = v[c * N + lin];
-        }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            php[a] = phi[nb_p[a]];
-            phm[a] = phi[nb_m[a]];
-            e2p[a] = e[(3 + a) * N + nb_p[a]];
-            v2p[a] = v[(3 + a) * N + nb_p[a]];
-            e1m[a] = e[a * N + nb_m[a]];
-            v1m[a] = v[a * N + nb_m[a]];
-        }
-        T eo[6], vo[6], fl[3], zz[6];
-        voxel_step<T, OUT>(K, ec, vc, gam[lin], phi[lin], php, phm, e2p, v2p, e1m, v1m, acc, eo, vo, fl,
-                           (!OUT && p.zout) ? zz : nullptr);
-        if (!OUT && p.zout) {
-            // the pre-projection point z = v + rho xi of this update, kept for the reverse pass
-            T* zo = p.zout + (size_t)s * 6 * N;
-#pragma unroll
-            for (int c = 0; c < 6; ++c) zo[c * N + lin] = zz[c];
-        }
-        if (OUT) {
-            if (p.cut) {
-                T* cut = p.cut + (size_t)s * 6 * N;
-#pragma unroll
-                for (int c = 0; c < 6; ++c) cut[c * N + lin] = eo[c];
-            }
-            if (p.flow) {
-                T* flow = p.flow + (size_t)s * 3 * N;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) flow[a * N + lin] = fl[a];
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                e_out[c * N + lin] = eo[c];
-                v_out[c * N + lin] = vo[c];
-            }
-        }
-    }
-    update_epilogue<T, OUT>(g, p, cfg, S, s, rho_d, acc);
-}
-
-// VW consecutive elements of the field type with one aligned load / store.
-template <typename T, int VW> struct VecN;
-template <> struct VecN<float, 4> {
-    __device__ __forceinline__ static void ld(const float* __restrict__ p, float (&o)[4]) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(p));
-        o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
-    }
-    __device__ __forceinline__ static void st(float* p, const float (&o)[4]) {
-        *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
-    }
-};
-template <> struct VecN<float, 2> {
-    __device__ __forceinline__ static void ld(const float* __restrict__ p, float (&o)[2]) {
-        const float2 t = __ldg(reinterpret_cast<const float2*>(p));
-        o[0] = t.x; o[1] = t.y;
-    }
-    __device__ __forceinline__ static void st(float* p, const float (&o)[2]) {
-        *reinterpret_cast<float2*>(p) = make_float2(o[0], o[1]);
-    }
-};
-template <> struct VecN<float, 1> {
-    __device__ __forceinline__ static void ld(const float* __restrict__ p, float (&o)[1]) { o[0] = __ldg(p); }
-    __device__ __forceinline__ static void st(float* p, const float (&o)[1]) { p[0] = o[0]; }
-};
-template <> struct VecN<double, 2> {
-    __device__ __forceinline__ static void ld(const double* __restrict__ p, double (&o)[2]) {
-        const double2 t = __ldg(reinterpret_cast<const double2*>(p));
-        o[0] = t.x; o[1] = t.y;
-    }
-    __device__ __forceinline__ static void st(double* p, const double (&o)[2]) {
-        *reinterpret_cast<double2*>(p) = make_double2(o[0], o[1]);
-    }
-};
-template <> struct VecN<double, 1> {
-    __device__ __forceinline__ static void ld(const double* __restrict__ p, double (&o)[1]) { o[0] = __ldg(p); }
-    __device__ __forceinline__ static void st(double* p, const double (&o)[1]) { p[0] = o[0]; }
-};
-
-// Vector version of the advancing update: W consecutive voxels of a z line per
-// thread, 16-byte loads and stores (N3 % W == 0, 16-byte aligned gamma). The
-// instantiation with half the voxels per thread (8-byte vectors in FP32) needs about
-// half the registers and runs two blocks per SM (update variant 11).
-template <typename T, bool OUT, int W = Vec16<T>::W, int MINB = 1>
-__global__ void __launch_bounds__(kThreads, MINB) k_update_vec(Geom g, Ptrs<T> p, LoopConfig cfg) {
-    using V = VecN<T, W>;
-    const int s = blockIdx.y + p.s0;
-    SolveScalars& S = p.sc[s];
-    if (!OUT && !S.active) return;
-    const long long N = g.N;
-    const double rho_d = S.rho;
-    const StepConsts<T> K = step_consts<T>(S, cfg);
-    const int par = S.iters & 1;
-    const T* __restrict__ e = p.e + (long long)par * p.sstride + (long long)s * 6 * N;
-    const T* __restrict__ v = p.v + (long long)par * p.sstride + (long long)s * 6 * N;
-    T* __restrict__ e_out = p.e + (long long)(1 - par) * p.sstride + (long long)s * 6 * N;
-    T* __restrict__ v_out = p.v + (long long)(1 - par) * p.sstride + (long long)s * 6 * N;
-    const T* __restrict__ phi = p.phi + (size_t)s * N;
-    const T* __restrict__ gam = gamma_of(p, s);
-    const long long ngroups = N / W;
-    // Dynamic schedule: blocks take chunks of kVecChunkGroups x kThreads groups (32 rows at
-    // N3 = 512) in order from a per-solve ticket counter, the next ticket fetched while the
-    // current chunk runs. The chunks in flight then form one narrow front through the grid, and
-    // the x- and y-neighbour rows a chunk reads were read as other chunks' own rows moments
-    // before, so they come from L2. (With a grid-stride loop the blocks drift apart over a long
-    // pass; at 512^3, 42 % more than the algorithmic reads came from DRAM.) Each chunk stores its
-    // own partial sums and the last block reduces them in chunk order, so the result does not
-    // depend on which block took which chunk.
-    const long long nchunks = vec_update_chunks(N, W);
-    double* part = p.partial + (size_t)s * nchunks * kNSum;
-    __shared__ unsigned ticket[2];
-    if (threadIdx.x == 0) ticket[0] = atomicAdd(&S.chunk, 1u);
-    __syncthreads();
-    for (int it = 0;; ++it) {
-        const unsigned ck = ticket[it & 1];
-        if (ck >= nchunks) break;   // the same value for the whole block
-        if (threadIdx.x == 0) ticket[(it + 1) & 1] = atomicAdd(&S.chunk, 1u);
-        T acc[kNSum];
-#pragma unroll
-        for (int q = 0; q < kNSum; ++q) acc[q] = T(0);
-#pragma unroll 1
-        for (int gi = 0; gi < kVecChunkGroups; ++gi) {
-            const long long q = ((long long)ck * kVecChunkGroups + gi) * kThreads + threadIdx.x;
-            if (q < ngroups) {
-                const long long lin0 = q * W;
-                const unsigned row = fdiv((unsigned)lin0, g.div_n3);
-                const int k0 = (int)(lin0 - (long long)row * g.n3);
-                const RowNb rn = row_neighbours(g, row);
-                const int kp = (k0 + W == g.n3) ? 0 : k0 + W;
-                const int km = (k0 == 0) ? g.n3 - 1 : k0 - 1;
-                T ec[6][W], vc[6][W];
-#pragma unroll
-                for (int c = 0; c < 6; ++c) {
-                    V::ld(e + c * N + lin0, ec[c]);
-                    V::ld(v + c * N + lin0, vc[c]);
-                }
-                T gm[W], ph[W];
-                V::ld(gam + lin0, gm);
-                V::ld(phi + lin0, ph);
-                // x and y neighbours (whole groups), z neighbours inside the group or one scalar each side
-                T e2x[W], v2x[W], e1x[W], v1x[W], e2y[W], v2y[W], e1y[W], v1y[W];
-                T phxp[W], phxm[W], phyp[W], phym[W];
-                V::ld(e + 3 * N + rn.ip + k0, e2x);
-                V::ld(v + 3 * N + rn.ip + k0, v2x);
-                V::ld(e + 0 * N + rn.im + k0, e1x);
-                V::ld(v + 0 * N + rn.im + k0, v1x);
-                V::ld(e + 4 * N + rn.jp + k0, e2y);
-                V::ld(v + 4 * N + rn.jp + k0, v2y);
-                V::ld(e + 1 * N + rn.jm + k0, e1y);
-                V::ld(v + 1 * N + rn.jm + k0, v1y);
-                V::ld(phi + rn.ip + k0, phxp);
-                V::ld(phi + rn.im + k0, phxm);
-                V::ld(phi + rn.jp + k0, phyp);
-                V::ld(phi + rn.jm + k0, phym);
-                const T e2z_after = __ldg(e + 5 * N + rn.row + kp), v2z_after = __ldg(v + 5 * N + rn.row + kp);
-                const T e1z_before = __ldg(e + 2 * N + rn.row + km), v1z_before = __ldg(v + 2 * N + rn.row + km);
-                const T ph_after = __ldg(phi + rn.row + kp), ph_before = __ldg(phi + rn.row + km);
-                T eo[6][W], vo[6][W], fo[3][W];
-#pragma unroll
-                for (int u = 0; u < W; ++u) {
-                    T ecu[6], vcu[6];
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) {
-                        ecu[c] = ec[c][u];
-                        vcu[c] = vc[c][u];
-                    }
-                    const bool last = (u + 1 == W), first = (u == 0);
-                    const T php[3] = {phxp[u], phyp[u], last ? ph_after : ph[(u + 1) % W]};
-                    const T phm[3] = {phxm[u], phym[u], first ? ph_before : ph[(u + W - 1) % W]};
-                    const T e2p[3] = {e2x[u], e2y[u], last ? e2z_after : ec[5][(u + 1) % W]};
-                    const T v2p[3] = {v2x[u], v2y[u], last ? v2z_after : vc[5][(u + 1) % W]};
-                    const T e1m[3] = {e1x[u], e1y[u], first ? e1z_before : ec[2][(u + W - 1) % W]};
-                    const T v1m[3] = {v1x[u], v1y[u], first ? v1z_before : vc[2][(u + W - 1) % W]};
-                    T eou[6], vou[6], fl[3];
-                    voxel_step<T, OUT>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou, fl);
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) {
-                        eo[c][u] = eou[c];
-                        vo[c][u] = vou[c];
-                    }
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) fo[a][u] = fl[a];
-                }
-                if (OUT) {
-                    // final evaluation: the cut xi^{K+1/2} and the flow A* v^K
-                    if (p.cut) {
-                        T* cut = p.cut + (size_t)s * 6 * N;
-#pragma unroll
-                        for (int c = 0; c < 6; ++c) V::st(cut + c * N + lin0, eo[c]);
-                    }
-                    if (p.flow) {
-                        T* flow = p.flow + (size_t)s * 3 * N;
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) V::st(flow + a * N + lin0, fo[a]);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) {
-                        V::st(e_out + c * N + lin0, eo[c]);
-                        V::st(v_out + c * N + lin0, vo[c]);
-                    }
-                }
-            }
-        }
-        block_store_partial<T, kNSum>(acc, part, ck);
-        __syncthreads();   // the next ticket is visible, this one is read by everyone, red[] is free
-    }
-    if (block_ticket(&S.counter, gridDim.x)) update_finish<T, OUT>(g, p, cfg, S, s, rho_d, part, (int)nchunks);
-}
-
 
 // ---------------------------------------------------------------------------
 // Stored-divergence schedule (update variants 8 and 9). By Eq. 28 and Eq. 30 the
@@ -1730,7 +1422,7 @@ __global__ void __launch_bounds__(AbVariant<T, VAR>::NW * 32, AbVariant<T, VAR>:
     const int n1 = g.n1, n2 = g.n2, n3 = g.n3;
     const double rho_d = S.rho;
     const StepConsts<T> K = step_consts<T>(S, cfg);
-    const T h = K.h;
+    const T h = div_scale<T>();   // the factor that the passes keep in a and b (see pass 1)
     const int par = S.iters & 1;
     const T* __restrict__ e = p.e + (long long)par * p.sstride + (long long)s * 6 * N;
     const T* __restrict__ v = p.v + (long long)par * p.sstride + (long long)s * 6 * N;
@@ -1992,7 +1684,7 @@ __global__ void __launch_bounds__(kAbwWarps * 32, MINB) k_update_abw(Geom g, Ptr
     const int n1 = g.n1, n2 = g.n2, n3 = g.n3;
     const double rho_d = S.rho;
     const StepConsts<T> K = step_consts<T>(S, cfg);
-    const T h = K.h;
+    const T h = div_scale<T>();   // the factor that the passes keep in a and b (see pass 1)
     const int par = S.iters & 1;
     const T* __restrict__ e = p.e + (long long)par * p.sstride + (long long)s * 6 * N;
     const T* __restrict__ v = p.v + (long long)par * p.sstride + (long long)s * 6 * N;
@@ -2184,7 +1876,6 @@ __global__ void __launch_bounds__(kThreads) k_ab_init(Geom g, Ptrs<T> p) {
     const SolveScalars& S = p.sc[s];
     if (S.ab_iter == S.iters) return;
     const long long N = g.N;
-    const T h = T(0.70710678118654752440084436210485);
     const long long cur = (long long)(S.iters & 1) * p.sstride + (long long)s * 6 * N;
     const T* __restrict__ e = p.e + cur;
     const T* __restrict__ v = p.v + cur;
@@ -2200,7 +1891,7 @@ __global__ void __launch_bounds__(kThreads) k_ab_init(Geom g, Ptrs<T> p) {
             const T sx = f[0 * N + lin] - f[0 * N + rn.im + k] + f[3 * N + rn.ip + k] - f[3 * N + lin];
             const T sy = f[1 * N + lin] - f[1 * N + rn.jm + k] + f[4 * N + rn.jp + k] - f[4 * N + lin];
             const T sz = f[2 * N + lin] - f[2 * N + rn.row + km] + f[5 * N + rn.row + kp] - f[5 * N + lin];
-            return h * (sx + sy + sz);
+            return div_scale<T>() * (sx + sy + sz);
         };
         a_out[lin] = dv(e);
         b_out[lin] = dv(v);

@@ -4,6 +4,7 @@
 #include "ccmf_kernels.cuh"
 #include "ccmf_persist.cuh"
 #include "ccmf_tma_x.cuh"
+#include "ccmf_update.cuh"
 
 namespace ccmf {
 
@@ -31,6 +32,7 @@ struct Ctx {
     LaunchShape sh;
     bool vec_div;         // 16-byte path of the divergence pass (N3 % W == 0)
     bool vec_update;      // 16-byte path of the update pass (also needs gamma 16-byte aligned)
+    bool use_zs;          // the update pass writes the (z, s) state (p.zs is the device's copy)
     bool use_ab;          // stored-divergence schedule: update variants 8 .. 10 write a, b; the first pass reads them
 };
 
@@ -176,23 +178,56 @@ int lines_blocks_per_sm(int mode, int lines, size_t smem) {
     return nb;
 }
 
-// Resident blocks per SM of the vector update pass (the smaller of the advancing and
-// the final-evaluation kernels), at least 1.
+// Instantiations of k_update: update variant 0 (16-byte vectors), 11 (half of them, two blocks per SM), 12
+// (half, three blocks per SM), any N3 or alignment (strided packs); FP32 writes the (z, s) format, or (e, v)
+// where the caller needs it (WZS = false, strided packs only: the reverse mode's forward passes and update variants
+// 1 .. 10, 13 .. 15 on grids that they do not cover). FP64 always writes (e, v).
+enum UpdateKind { kUpdFull = 0, kUpdHalf2, kUpdHalf3, kUpdStrided, kUpdStridedEv, kNumUpdateKinds };
+
+template <typename T, bool OUT, int RULE>
+const void* update_kernel(int kind) {
+    constexpr bool F = sizeof(T) == 4;
+    constexpr int WF = Vec16<T>::W;
+    constexpr int WH = F ? 2 : 0;   // one FP64 voxel is a strided pack
+    if constexpr (OUT) {
+        return kind == kUpdFull ? (const void*)k_update<T, WF, true, -1, F, 1>
+                                : (const void*)k_update<T, 0, true, -1, F, 1>;
+    } else {
+        switch (kind) {
+            case kUpdFull: return (const void*)k_update<T, WF, false, RULE, F, 1>;
+            case kUpdHalf2: return (const void*)k_update<T, WH, false, RULE, F, 2>;
+            case kUpdHalf3: return (const void*)k_update<T, WH, false, RULE, F, 3>;
+            case kUpdStrided: return (const void*)k_update<T, 0, false, RULE, F, 2>;
+            default: return (const void*)k_update<T, 0, false, -1, false, 2>;
+        }
+    }
+}
+
+// Voxels of a thread group of an update kernel.
 template <typename T>
-int update_vec_blocks_per_sm() {
-    int a = 0, b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_update_vec<T, false>, kThreads, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_update_vec<T, true>, kThreads, 0) != cudaSuccess) {
+constexpr int update_voxels(int kind) {
+    return kind == kUpdFull ? Vec16<T>::W : sizeof(T) == 4 ? 2 : 1;
+}
+
+// Resident blocks per SM of an update kernel, at least 1.
+template <typename T>
+int update_blocks_per_sm(int kind, bool out) {
+    int a = 0;
+    const void* f = out ? update_kernel<T, true, -1>(kind) : update_kernel<T, false, -1>(kind);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, f, kThreads, 0) != cudaSuccess) {
         cudaGetLastError();
         return 1;
     }
-    const int m = a < b ? a : b;
-    return m < 1 ? 1 : m;
+    return a < 1 ? 1 : a;
 }
 
-// Update variant 11: the vector update pass with half the voxels per thread, two blocks per SM.
+// The kernel of the register update pass of a context.
 template <typename T>
-constexpr int kVecHalfW = Vec16<T>::W / 2;
+int update_kind(const Ctx<T>& c) {
+    if (sizeof(T) == 4 && !c.use_zs) return kUpdStridedEv;
+    if (!c.vec_update) return kUpdStrided;
+    return c.sh.upd_variant == 11 ? kUpdHalf2 : c.sh.upd_variant == 12 ? kUpdHalf3 : kUpdFull;
+}
 
 #define CCMF_DISPATCH_ABW(var, ...)                                                      \
     do {                                                                                 \
@@ -207,22 +242,6 @@ constexpr int kVecHalfW = Vec16<T>::W / 2;
             __VA_ARGS__;                                                                 \
         }                                                                                \
     } while (0)
-
-// Resident blocks per SM of update variant 11 (12: the same vectors, three blocks per SM), at
-// least 1.
-template <typename T>
-int update_vec_half_blocks_per_sm(int variant) {
-    int a = 0;
-    const cudaError_t e =
-        variant == 12
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_update_vec<T, false, kVecHalfW<T>, 3>, kThreads, 0)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_update_vec<T, false, kVecHalfW<T>, 2>, kThreads, 0);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return 1;
-    }
-    return a < 1 ? 1 : a;
-}
 
 // Blocks per SM of a warp-per-line pass of length n (power of two 128 ... 1024), 0 on error.
 template <typename T>
@@ -363,6 +382,13 @@ template <typename T>
 void launch_init(const Ctx<T>& c, cudaStream_t st) {
     k_setup<T><<<(unsigned)ceil_div(c.g.batch, 128), 128, 0, st>>>(c.p.sc, c.xi_stage, c.g.batch);
     dim3 grid((unsigned)c.sh.grid_update, (unsigned)c.g.batch);
+    if constexpr (sizeof(T) == 4) {
+        if (c.cfg.resume && !c.p.zs) {
+            // a state that a (z, s) plan left, for passes that read (e, v)
+            k_state_to_ev<T><<<grid, kThreads, 0, st>>>(c.g, c.p, 0);
+            k_state_mark_ev<T><<<(unsigned)ceil_div(c.g.batch, 128), 128, 0, st>>>(c.p.sc, c.g.batch);
+        }
+    }
     k_init_stats<T><<<grid, kThreads, 0, st>>>(c.g, c.p, c.cfg);
     if (!c.cfg.resume) k_init_state<T><<<grid, kThreads, 0, st>>>(c.g, c.p);
     if (c.use_ab) k_ab_init<T><<<grid, kThreads, 0, st>>>(c.g, c.p);
@@ -416,12 +442,15 @@ void launch_passes(const Ctx<T>& c, const Ptrs<T>& p, cudaStream_t st, F&& betwe
     if (sh.grid_x > 0 && sh.grid_x < twx) twx = sh.grid_x;
     dim3 gwy((unsigned)twy, (unsigned)g.batch);
     dim3 gwx((unsigned)twx, (unsigned)g.batch);
-    dim3 gu((unsigned)sh.grid_update, (unsigned)g.batch);
-    // the vector update pass takes its chunks from a ticket counter: the resident blocks, shared
+    // the register update pass takes its chunks from a ticket counter: the resident blocks, shared
     // by the solves of this launch, so that every solve's chunks run at once on all SMs
-    const int vpb = sh.vec_resident > 0 ? sh.vec_resident / g.batch : sh.grid_update;
-    const dim3 gv((unsigned)(vpb < 1 ? 1 : vpb), (unsigned)g.batch);
-    const T inv_n = (T)(1.0 / (double)g.N);
+    auto grid_upd = [&](int resident, int kind) {
+        const long long chunks = vec_update_chunks<T>(g.N, update_voxels<T>(kind));
+        long long b = resident > 0 ? resident / g.batch : sh.grid_update;
+        b = b < chunks ? b : chunks;
+        return dim3((unsigned)(b < 1 ? 1 : b), (unsigned)g.batch);
+    };
+    const T inv_n = (T)(poisson_scale<T>() / (double)g.N);
     const dim3 gwz((unsigned)ceil_div((long long)g.n1 * g.n2, 2 * (kThreads / 32)), (unsigned)g.batch);
     const bool ab = !OUT && c.use_ab;   // the first pass reads the stored divergences a, b
     if (sh.wzd && c.vec_div) {
@@ -513,11 +542,11 @@ void launch_passes(const Ctx<T>& c, const Ptrs<T>& p, cudaStream_t st, F&& betwe
                             { k_irfft_z<T, LN><<<gzi, kThreads, sh.smem_zi, st>>>(g, p, c.ax[2], c.tw[2]); });
     }
     between(kKIrfftZ);
-    if (OUT && c.vec_update && vec_out_ok(p))
-        k_update_vec<T, true><<<gv, kThreads, 0, st>>>(g, p, c.cfg);
-    else if (OUT)
-        k_update<T, true><<<gu, kThreads, 0, st>>>(g, p, c.cfg);
-    else if (ab && is_abw_variant(sh.upd_variant)) {
+    void* uargs[] = {(void*)&g, (void*)&p, (void*)&c.cfg};
+    if (OUT) {
+        const int kind = c.vec_update && vec_out_ok(p) ? kUpdFull : kUpdStrided;
+        cudaLaunchKernel(update_kernel<T, true, -1>(kind), grid_upd(sh.out_resident, kind), dim3(kThreads), uargs, 0, st);
+    } else if (ab && is_abw_variant(sh.upd_variant)) {
         const long long items = (long long)sh.ab.nq * sh.ab.nr * sh.ab.npass;
         const dim3 ga((unsigned)ceil_div(items, kAbwWarps), (unsigned)g.batch);
         CCMF_DISPATCH_ABW(sh.upd_variant, {
@@ -547,17 +576,12 @@ void launch_passes(const Ctx<T>& c, const Ptrs<T>& p, cudaStream_t st, F&& betwe
         else
             k_update_tma<T, 1><<<gt, kThreads, sh.smem_tma, st>>>(g, p, c.cfg, sh.tma_rows);
     }
-    else if (c.vec_update && (sh.upd_variant == 11 || sh.upd_variant == 12)) {
-        const int vpb2 = sh.vec_resident_half > 0 ? sh.vec_resident_half / g.batch : sh.grid_update;
-        const dim3 gv2((unsigned)(vpb2 < 1 ? 1 : vpb2), (unsigned)g.batch);
-        if (sh.upd_variant == 12)
-            k_update_vec<T, false, kVecHalfW<T>, 3><<<gv2, kThreads, 0, st>>>(g, p, c.cfg);
-        else
-            k_update_vec<T, false, kVecHalfW<T>, 2><<<gv2, kThreads, 0, st>>>(g, p, c.cfg);
-    } else if (c.vec_update)
-        k_update_vec<T, false><<<gv, kThreads, 0, st>>>(g, p, c.cfg);
-    else
-        k_update<T, false><<<gu, kThreads, 0, st>>>(g, p, c.cfg);
+    else {
+        const int kind = update_kind(c);
+        const bool bb = c.cfg.rho_rule == 0 || c.cfg.rho_rule == 3;   // the other rules' sums are not needed
+        cudaLaunchKernel(bb ? update_kernel<T, false, 0>(kind) : update_kernel<T, false, -1>(kind),
+                         grid_upd(sh.upd_resident, kind), dim3(kThreads), uargs, 0, st);
+    }
     between(kKUpdate);
 }
 
@@ -596,6 +620,16 @@ void launch_final(const Ctx<T>& c, cudaStream_t st, T* cut, T* flow) {
     launch_passes<T, true>(c, p, st, NoHook());
 }
 
+// The current state of every solve as (e, v) in the other copy of the state buffers (FP32 plans; solves whose
+// state is in the (e, v) format already are left alone).
+template <typename T>
+void launch_expand_state(const Ctx<T>& c, cudaStream_t st) {
+    if constexpr (sizeof(T) == 4) {
+        dim3 grid((unsigned)c.sh.grid_update, (unsigned)c.g.batch);
+        k_state_to_ev<T><<<grid, kThreads, 0, st>>>(c.g, c.p, 1);
+    }
+}
+
 // ---- reverse mode (adjoint) helpers ------------------------------------------
 template <typename T>
 __global__ void k_adj_restore(SolveScalars* sc, int batch, int k0, const double* __restrict__ sched, int sched_len) {
@@ -607,6 +641,7 @@ __global__ void k_adj_restore(SolveScalars* sc, int batch, int k0, const double*
     sc[s].active = 1;
     sc[s].counter = 0;
     sc[s].chunk = 0;
+    sc[s].zs_iter = -1;
 }
 
 template <typename T>
@@ -615,6 +650,7 @@ __global__ void k_adj_dummy(SolveScalars* sc, int batch) {
     if (s >= batch) return;
     SolveScalars z = {};
     z.rho = 1.0;   // w = e - v / rho with e = y, v = 0: the passes apply M to y
+    z.zs_iter = -1;
     sc[s] = z;
 }
 

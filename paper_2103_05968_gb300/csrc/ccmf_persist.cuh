@@ -53,7 +53,7 @@ struct PersistGroup {
     const T* rsym_y;            // the same for y (the order pass 1 leaves)
     const T* sym_z;             // 4 sin^2(pi k / n3), natural order
     FastDiv div_l;              // the tile's line count L (in-place stage indexing)
-    T inv_n;                    // 1 / N
+    T inv_n;                    // poisson_scale / N
     int vec_div;                // pass 0 reads 16-byte vectors (n3 % (16 / sizeof(T)) == 0)
     int upd_w;                  // voxels per thread group of pass 5 (vector width)
     long long nchunks;          // pass-5 chunks per solve
@@ -134,7 +134,6 @@ __device__ void persist_div_rfft_z(const PersistGroup<T>& G, int s, long long t,
     C* A = reinterpret_cast<C*>(work);
     C* B = A + (size_t)g.n3 * stride;
     const T irho = T(1) / (T)p.sc[s].rho;
-    const T h = T(0.70710678118654752440084436210485);
     const long long N = g.N;
     const long long cur = (long long)(p.sc[s].iters & 1) * p.sstride + (long long)s * 6 * N;
     const T* __restrict__ e = p.e + cur;
@@ -190,7 +189,7 @@ __device__ void persist_div_rfft_z(const PersistGroup<T>& G, int s, long long t,
                     const T sx = w[0][u] - xm[u] + xp[u] - w[3][u];
                     const T sy = w[1][u] - ym[u] + yp[u] - w[4][u];
                     const T sz = w[2][u] - w1zm + w2zp - w[5][u];
-                    d[u] = h * (sx + sy + sz);
+                    d[u] = div_scale<T>() * (sx + sy + sz);
                 }
             } else {
                 const long long p0 = rn.row + k0;
@@ -198,7 +197,7 @@ __device__ void persist_div_rfft_z(const PersistGroup<T>& G, int s, long long t,
                 const T sx = wc(0, p0) - wc(0, rn.im + k0) + wc(3, rn.ip + k0) - wc(3, p0);
                 const T sy = wc(1, p0) - wc(1, rn.jm + k0) + wc(4, rn.jp + k0) - wc(4, p0);
                 const T sz = wc(2, p0) - wc(2, rn.row + km) + wc(5, rn.row + kp) - wc(5, p0);
-                d[0] = h * (sx + sy + sz);
+                d[0] = div_scale<T>() * (sx + sy + sz);
             }
         }
 #pragma unroll
@@ -288,7 +287,7 @@ __device__ void persist_x_lines(const PersistGroup<T>& G, int s, long long t, co
     const T lam23 = valid ? G.rsym_y[k2] + G.sym_z[kz] : T(0);
     for (int m = m0; m < n; m += mstep) {
         const T lam = G.rsym_x[m] + lam23;
-        const T gk = (valid && lam > T(0)) ? -G.inv_n / lam : T(0);
+        const T gk = (valid && lam > T(0)) ? poisson_gain_div(G.inv_n, lam) : T(0);
         const C z = b[m * stride + cl];
         b[m * stride + cl] = cmake<C>(z.x * gk, -z.y * gk);
     }
@@ -356,8 +355,14 @@ __device__ void persist_irfft_z(const PersistGroup<T>& G, int s, long long t, co
     }
 }
 
-// Pass 5 on chunk ck: kVecChunkGroups x kThreads groups of W consecutive voxels of a z line
-// (as the chunks of k_update_vec); stores the chunk's partial sums in slot ck.
+// Pass 5 on chunk ck: kPersistChunkGroups x kThreads groups of W consecutive voxels of a z line; stores the
+// chunk's partial sums in slot ck. (A chunk is one work item here, so its size does not follow the grid.)
+constexpr int kPersistChunkGroups = 16;
+__host__ __device__ inline long long persist_chunks(long long n_voxels, int voxels_per_group) {
+    const long long per = (long long)kThreads * kPersistChunkGroups * voxels_per_group;
+    return (n_voxels + per - 1) / per;
+}
+
 template <typename T, int W>
 __device__ void persist_update(const PersistGroup<T>& G, int s, long long ck, const LoopConfig& cfg) {
     using V = VecN<T, W>;
@@ -379,8 +384,8 @@ __device__ void persist_update(const PersistGroup<T>& G, int s, long long ck, co
 #pragma unroll
     for (int q = 0; q < kNSum; ++q) acc[q] = T(0);
 #pragma unroll 1
-    for (int gi = 0; gi < kVecChunkGroups; ++gi) {
-        const long long q = (ck * kVecChunkGroups + gi) * kThreads + threadIdx.x;
+    for (int gi = 0; gi < kPersistChunkGroups; ++gi) {
+        const long long q = (ck * kPersistChunkGroups + gi) * kThreads + threadIdx.x;
         if (q >= ngroups) break;
         const long long lin0 = q * W;
         const unsigned row = fdiv((unsigned)lin0, g.div_n3);

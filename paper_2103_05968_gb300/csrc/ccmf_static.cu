@@ -175,7 +175,8 @@ int static_solve(int n1, int n2, int n3, const T* gamma, const double* xi_bar, c
     sh.smem_x = ((size_t)n1 + 2 * (size_t)n1 * (sh.lpb_x + 1)) * cs;
     long long gu = (g.N + kThreads - 1) / kThreads;
     sh.grid_update = (int)(gu < kStaticGridUpdate ? gu : kStaticGridUpdate);
-    sh.vec_resident = 0;   // the vector update pass runs grid_update blocks per solve
+    sh.upd_resident = sh.out_resident = 0;   // the update pass runs grid_update blocks per solve
+    sh.upd_variant = sizeof(T) == 4 ? 12 : 0;
 
     // scratch layout: scalars, counter, normal, partials, history, state (two copies),
     // spectrum, phi, tables
@@ -187,9 +188,14 @@ int static_solve(int n1, int n2, int n3, const T* gamma, const double* xi_bar, c
         return o;
     };
     const size_t o_sc = take(256), o_nact = take(256), o_xi = take(3 * sizeof(double));
-    // partial sums: one slot per update block, or per chunk of the vector update pass
-    const long long nparts = std::max<long long>(sh.grid_update, vec_update_chunks(g.N, 16 / (int)sizeof(T)));
-    const size_t o_part = take(sizeof(double) * kNSum * (size_t)nparts);
+    // partial sums: one slot per block of the voxel passes, or per chunk of the update pass (w voxels per thread
+    // group). Where the chunks are more than the blocks they go to the half spectrum, which no pass needs while
+    // the update runs, so that the scratch area fits the same grids whatever the chunk size.
+    long long nparts = 0;
+    for (int w = sizeof(T) == 4 ? 2 : 1; w <= 16 / (int)sizeof(T); w *= 2)
+        nparts = std::max<long long>(nparts, vec_update_chunks<T>(g.N, w));
+    const bool parts_in_spec = nparts > sh.grid_update;
+    const size_t o_part = take(sizeof(double) * kNSum * (size_t)sh.grid_update);
     const size_t o_hist = take(sizeof(double) * kHistFields * (size_t)kHistCap);
     const size_t o_e = take(sizeof(T) * 6 * N * 2), o_v = take(sizeof(T) * 6 * N * 2);
     const size_t o_spec = take(cs * (size_t)g.Nh), o_phi = take(sizeof(T) * N);
@@ -198,7 +204,9 @@ int static_solve(int n1, int n2, int n3, const T* gamma, const double* xi_bar, c
     for (int a = 0; a < 3; ++a) o_sy[a] = take(sizeof(T) * (size_t)nn[a]);
     size_t o_rs[2];
     for (int a = 0; a < 2; ++a) o_rs[a] = take(sizeof(T) * (size_t)nn[a]);
-    if (off > kStaticScratchBytes) return CCMF_ERR_UNSUPPORTED_SIZE;
+    if (off > kStaticScratchBytes ||
+        (parts_in_spec && sizeof(double) * kNSum * (size_t)nparts > cs * (size_t)g.Nh))
+        return CCMF_ERR_UNSUPPORTED_SIZE;
 
     unsigned char* ws = nullptr;
     int rc = static_setup(dev, &ws);
@@ -226,7 +234,7 @@ int static_solve(int n1, int n2, int n3, const T* gamma, const double* xi_bar, c
     c.xi_stage = reinterpret_cast<const double*>(ws + o_xi);
     c.p.sc = reinterpret_cast<SolveScalars*>(ws + o_sc);
     c.p.n_active = reinterpret_cast<int*>(ws + o_nact);
-    c.p.partial = reinterpret_cast<double*>(ws + o_part);
+    c.p.partial = reinterpret_cast<double*>(ws + (parts_in_spec ? o_spec : o_part));
     c.p.hist = reinterpret_cast<double*>(ws + o_hist);
     c.p.e = reinterpret_cast<T*>(ws + o_e);
     c.p.v = reinterpret_cast<T*>(ws + o_v);
@@ -238,6 +246,8 @@ int static_solve(int n1, int n2, int n3, const T* gamma, const double* xi_bar, c
     const int W = 16 / (int)sizeof(T);
     c.vec_div = (n3 % W) == 0;
     c.vec_update = c.vec_div && ((uintptr_t)gamma % 16) == 0;
+    c.use_zs = sizeof(T) == 4;
+    c.p.zs = c.use_zs ? 1 : 0;
 
     // clear what must start from a known value: the active counter, the history ring
     const double nn2 = xi_bar[0] * xi_bar[0] + xi_bar[1] * xi_bar[1] + xi_bar[2] * xi_bar[2];

@@ -25,13 +25,27 @@ constexpr int kHistFields = 6;
 constexpr int kHistCap = 4096;   // history entries reserved per solve
 constexpr int kThreads = 256;
 
-// The vector update pass works in chunks of kVecChunkGroups groups of 16 bytes per
-// thread (16 K voxels in FP32), taken in order from a ticket counter, with one
-// partial-sum slot per chunk.
+// The register update pass works in chunks, taken in order, with one partial-sum slot per chunk. A chunk is
+// kVecChunkGroups groups per thread (8 K voxels in FP32 with two voxels per group) on large grids. Grids that would give
+// fewer than kVecMinChunks chunks halve it until they do, so that the chunks spread over the SMs: 16 groups
+// give a 32^3 FP64 solve 4 chunks, i.e. 4 busy SMs (436 us a pass). In FP32 400 chunks were the best of 96, 400
+// and 1300 (96^3 x 6: 98 / 88 / 118 us a pass, 128^3 x 3: 194 / 185 / 202 us an iteration); in FP64, where a chunk's
+// arithmetic is long, 1300 (128^3: 735 / 741 / 700 us). The rule depends on the grid and the precision alone, so a
+// solve sums in the same order alone and in a batch.
 constexpr int kVecChunkGroups = 16;
+template <typename T>
+__host__ __device__ inline int vec_chunk_groups(long long n_voxels, int voxels_per_group) {
+    constexpr long long kVecMinChunks = sizeof(T) == 4 ? 400 : 1300;
+    const long long per_block = (long long)kThreads * voxels_per_group;
+    const long long groups = (n_voxels + per_block - 1) / per_block;
+    int per = kVecChunkGroups;
+    while (per > 1 && groups < kVecMinChunks * per) per /= 2;
+    return per;
+}
+template <typename T>
 __host__ __device__ inline long long vec_update_chunks(long long n_voxels, int voxels_per_group) {
-    const long long per = (long long)kThreads * kVecChunkGroups;
-    return (n_voxels / voxels_per_group + per - 1) / per;
+    const long long per = (long long)kThreads * voxels_per_group * vec_chunk_groups<T>(n_voxels, voxels_per_group);
+    return (n_voxels + per - 1) / per;
 }
 
 // One per solve, in the workspace (256-byte slot).
@@ -50,6 +64,8 @@ struct SolveScalars {
     int bad;             // number of invalid gamma values seen at init
     unsigned int chunk;  // next work ticket of the vector update pass (dynamic schedule)
     int ab_iter;         // update count the stored divergences a, b belong to (-1: not current)
+    int zs_iter;         // update count of a state in the (z, s) format (FP32; any other value: (e, v))
+    double rho_prev;     // the penalty of the update that wrote the (z, s) state
 };
 static_assert(sizeof(SolveScalars) <= 256, "scalar slot");
 
@@ -76,8 +92,8 @@ struct Ptrs {
     int* n_active;
     double* partial;      // [batch][grid_update][kNSum]
     double* hist;         // [batch][hist_len][kHistFields]
-    T* e;                 // [2][batch][6][N]: two copies, the current one is (iters & 1)
-    T* v;                 // [2][batch][6][N]
+    T* e;                 // [2][batch][6][N]: two copies, the current one is (iters & 1); z in the (z, s) format
+    T* v;                 // [2][batch][6][N]; s in the first component in the (z, s) format
     long long sstride;    // elements between the two copies (batch * 6 * N)
     cx<T>* spec;          // [batch][Nh]
     T* phi;               // [batch][N]
@@ -88,7 +104,8 @@ struct Ptrs {
     T* flow;              // [batch][3][N] (final pass, may be null)
     int run_all;          // 1: passes run for every solve (final evaluation), 0: active solves only
     int s0;               // first solve of this launch (blockIdx.y counts from it)
-    T* zout;              // when not null the (scalar) update pass also writes z = v + rho xi, [batch][6][N]
+    T* zout;              // when not null an (e, v)-format update also writes z = v + rho xi, [batch][6][N]
+    int zs;               // 1: the update pass of this plan writes the (z, s) format (FP32)
     T* ab;                // stored divergences a = div^- A* e, b = div^- A* v of the state, [batch][2][N]
 };
 
@@ -109,8 +126,8 @@ struct LaunchShape {
     size_t smem_zi;           // its dynamic shared memory
     int lpb_y, lpb_x;         // strided passes: lines per block
     int grid_update;          // blocks per solve of the voxel passes
-    int vec_resident;         // resident blocks of the vector update pass on the whole GPU
-    int vec_resident_half;    // the same for update variants 11, 12 (fewer voxels per thread)
+    int upd_resident;         // resident blocks of the register update pass (variants 0, 11, 12) on the whole GPU
+    int out_resident;         // the same of the final evaluation pass
     size_t smem_z, smem_y, smem_x;
     int tma_rows;             // TMA-staged update: z rows per tile (0 = path not available)
     int grid_tma;             // blocks per solve of the TMA-staged update
