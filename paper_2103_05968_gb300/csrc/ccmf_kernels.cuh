@@ -11,13 +11,13 @@
 //                       (the (div^- grad^+)^+ of Eq. 28), inverse FFT along x;
 //   4. k_fft_lines<2>   inverse FFT along y;
 //   5. k_irfft_z        complex-to-real inverse FFT along z -> phi;
-//   6. k_update         xi^{k+1/2} = w - A(A* w - grad^+ phi - xi_bar) (= P_K(w),
+//   6. k_update<false>  xi^{k+1/2} = w - A(A* w - grad^+ phi - xi_bar) (= P_K(w),
 //                       Eq. 28), over-relaxation, z = v + rho xi, node-wise
 //                       projection onto C_gamma (Eq. 19), e^{k+1}, v^{k+1}
 //                       (Eq. 30), block partial sums; the last block reduces
 //                       them in double and updates rho, the history and the stop
 //                       flag on the device (Eq. 31, BB / LTD scaling).
-// (ccmf_update.cuh.) Its OUT instantiation is the final evaluation: it writes the cut xi^{K+1/2} and the
+// k_update<true> is the final evaluation: it writes the cut xi^{K+1/2} and the
 // flow A* v^K instead of advancing the state.
 #pragma once
 
@@ -337,11 +337,11 @@ __global__ void __launch_bounds__(kThreads) k_init_state(Geom g, Ptrs<T> p) {
 // VEC: each thread reads W consecutive voxels of a line with 16-byte loads.
 // ---------------------------------------------------------------------------
 template <typename T, int P, bool VEC, bool AB = false>
-__global__ void __launch_bounds__(kThreads) k_div_rfft_z(Geom g, Ptrs<T> p, AxisPlan az,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 1) k_div_rfft_z(Geom g, Ptrs<T> p, AxisPlan az,
                                                          const cx<T>* __restrict__ tw) {
     using C = cx<T>;
     constexpr int stride = P + 1;
-    constexpr int W = VEC ? Vec16<T>::W : 1;
+    constexpr int W = !VEC ? 1 : AB ? Vec16<T>::W : kDivW;
     const int s = blockIdx.y + p.s0;
     if (!p.run_all && !p.sc[s].active) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -358,12 +358,11 @@ __global__ void __launch_bounds__(kThreads) k_div_rfft_z(Geom g, Ptrs<T> p, Axis
     const long long L = (long long)g.n1 * g.n2;
     const long long l0 = (long long)blockIdx.x * 2 * P;
     for (int t = threadIdx.x; t < g.n3; t += kThreads) twl[t] = tw[t];
-    const int n3w = g.n3 / W;
-    const int cnt = 2 * P * n3w;
+    const int cnt = 2 * P * g.n3 / W;
     T* Ar = reinterpret_cast<T*>(A);
     for (int idx = threadIdx.x; idx < cnt; idx += kThreads) {
-        const int ll = idx / n3w;
-        const int k0 = (idx - ll * n3w) * W;
+        const int ll = (int)fdiv((unsigned)(idx * W), g.div_n3);
+        const int k0 = idx * W - ll * g.n3;
         const long long l = l0 + ll;
         T d[W];
 #pragma unroll
@@ -373,8 +372,8 @@ __global__ void __launch_bounds__(kThreads) k_div_rfft_z(Geom g, Ptrs<T> p, Axis
             const T* a = p.ab + (size_t)s * 2 * N + l * g.n3 + k0;
             if constexpr (VEC) {
                 T ta[W], tb[W];
-                Vec16<T>::ld(a, ta);
-                Vec16<T>::ld(a + N, tb);
+                VecN<T, W>::ld(a, ta);
+                VecN<T, W>::ld(a + N, tb);
 #pragma unroll
                 for (int u = 0; u < W; ++u) d[u] = ta[u] - tb[u] * irho;
             } else {
@@ -385,9 +384,9 @@ __global__ void __launch_bounds__(kThreads) k_div_rfft_z(Geom g, Ptrs<T> p, Axis
             const int kp = (k0 + W == g.n3) ? 0 : k0 + W;      // first voxel after the group
             const int km = (k0 == 0) ? g.n3 - 1 : k0 - 1;        // last voxel before the group
             auto div = [&](auto fmt) {
-                if constexpr (VEC)
+                if constexpr (VEC && !AB)
                     div_group<T, decltype(fmt)::value>(f, rn, k0, kp, km, d);
-                else
+                else if constexpr (!VEC)
                     d[0] = div_voxel<T, decltype(fmt)::value>(f, rn, k0, kp, km);
             };
             if constexpr (sizeof(T) == 4) {
@@ -941,8 +940,8 @@ __global__ void __launch_bounds__(kThreads, wz_min_blocks<T, N>())
     const long long l0 = (long long)blockIdx.x * RL;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     C* x = lines + w * LS;
-    // each lane takes groups of W consecutive z (16-byte loads), groups 32 W apart
-    constexpr int W = Vec16<T>::W;
+    // each lane takes groups of W consecutive z, groups 32 W apart
+    constexpr int W = AB ? Vec16<T>::W : kDivW;
     constexpr int G = N / (32 * W);      // groups per lane
     static_assert(G >= 1, "line too short for the warp z pass");
     // Group by group, both lines of the pair: a line's y-neighbour rows are the other line of
@@ -971,14 +970,15 @@ __global__ void __launch_bounds__(kThreads, wz_min_blocks<T, N>())
                 // stored divergences of the state: d = a - b / rho
                 const T* a = p.ab + (size_t)s * 2 * Nv + rn.row + k0;
                 T ta[W], tb[W];
-                Vec16<T>::ld(a, ta);
-                Vec16<T>::ld(a + Nv, tb);
+                VecN<T, W>::ld(a, ta);
+                VecN<T, W>::ld(a + Nv, tb);
 #pragma unroll
                 for (int u = 0; u < W; ++u) d[u] = ta[u] - tb[u] * irho;
             } else if (valid) {
                 const int kp = (k0 + W == N) ? 0 : k0 + W;   // first voxel after the group
                 const int km = (k0 == 0) ? N - 1 : k0 - 1;   // last voxel before the group
-                if constexpr (sizeof(T) == 4) {
+                if constexpr (AB) {
+                } else if constexpr (sizeof(T) == 4) {
                     if (zs)
                         div_group<T, true>(f, rn, k0, kp, km, d);
                     else

@@ -311,76 +311,68 @@ struct Group {
     }
 };
 
-// Pass 1's divergence d = div^- A* (e - v / rho) (Sec. 2.2, Eq. 17) of W consecutive voxels of a z row, with
-// 16-byte loads: d(p) = (1/sqrt2) sum_a [w1_a(p) - w1_a(p - e_a) + w2_a(p + e_a) - w2_a(p)]. kp / km: the voxels
-// just after / before the group (periodic).
+// Pass 1's divergence d = div^- A* (e - v / rho) (Sec. 2.2, Eq. 17) of kDivW consecutive voxels of a z row, with
+// vector loads: d(p) = (1/sqrt2) sum_a [w1_a(p) - w1_a(p - e_a) + w2_a(p + e_a) - w2_a(p)]. kp / km: the voxels
+// just after / before the group (periodic). Two voxels per thread: all loads of a group then fit 64 registers
+// and are in flight at once in four blocks per SM.
+constexpr int kDivW = 2;
+
 template <typename T, bool ZS>
 __device__ __forceinline__ void div_group(const StateSrc<T>& f, const RowNb& rn, int k0, int kp, int km,
-                                          T (&d)[Vec16<T>::W]) {
+                                          T (&d)[kDivW]) {
     using P = Pk<T>;
     using V = typename P::V;
-    constexpr int W = Vec16<T>::W;
-    using G = Group<T, W>;
+    using G = Group<T, kDivW>;
     constexpr int NP = G::NP;
     const long long N = f.N;
-    auto row_w = [&](int c, long long o, const V (&s)[NP], V (&w)[NP]) {
-        V x[NP], y[NP], e, v;
-        const typename G::Off off = {{o}};
-        G::ld(f.a + c * N, off, x);
-        if constexpr (!ZS) G::ld(f.b + c * N, off, y);
+    const typename G::Off own = {{rn.row + k0}};
+    const typename G::Off om[2] = {{{rn.im + k0}}, {{rn.jm + k0}}}, op[2] = {{{rn.ip + k0}}, {{rn.jp + k0}}};
+    // x, y: what the format stores of a component (z_c and s, or e_c and v_c)
+    V x0[6][NP], y0[ZS ? 1 : 6][NP], xm[2][NP], ym[2][NP], xp[2][NP], yp[2][NP];
 #pragma unroll
-        for (int q = 0; q < NP; ++q) state_evw<T, ZS>(f, x[q], ZS ? s[q] : y[q], e, v, w[q]);
-    };
-    auto row_s = [&](long long o, V (&s)[NP]) {
-        if constexpr (ZS) {
-            const typename G::Off off = {{o}};
-            G::ld(f.b, off, s);
-        }
-    };
-    const long long o = rn.row + k0;
-    V s0[NP], s1[NP], w[NP], n[NP], acc[NP];
-    row_s(o, s0);
-    // x and y: w1_a(p) - w1_a(p - e_a) + w2_a(p + e_a) - w2_a(p)
+    for (int c = 0; c < 6; ++c) G::ld(f.a + c * N, own, x0[c]);
+#pragma unroll
+    for (int c = 0; c < (ZS ? 1 : 6); ++c) G::ld(f.b + c * N, own, y0[c]);
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-        const long long om = (a == 0 ? rn.im : rn.jm) + k0, op = (a == 0 ? rn.ip : rn.jp) + k0;
-        V t[NP];
-        row_w(a, o, s0, w);
-        row_s(om, s1);
-        row_w(a, om, s1, n);
-#pragma unroll
-        for (int q = 0; q < NP; ++q) t[q] = P::sub(w[q], n[q]);
-        row_w(3 + a, o, s0, w);
-        row_s(op, s1);
-        row_w(3 + a, op, s1, n);
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            t[q] = P::sub(P::add(t[q], n[q]), w[q]);
-            acc[q] = a == 0 ? t[q] : P::add(acc[q], t[q]);
-        }
+        G::ld(f.a + a * N, om[a], xm[a]);
+        G::ld(ZS ? f.b : f.b + a * N, om[a], ym[a]);
+        G::ld(f.a + (3 + a) * N, op[a], xp[a]);
+        G::ld(ZS ? f.b : f.b + (3 + a) * N, op[a], yp[a]);
     }
-    // z: the neighbours inside the group, or one voxel on each side of it
     const T xa = __ldg(f.a + 5 * N + rn.row + kp), ya = __ldg((ZS ? f.b : f.b + 5 * N) + rn.row + kp);
     const T xb = __ldg(f.a + 2 * N + rn.row + km), yb = __ldg((ZS ? f.b : f.b + 2 * N) + rn.row + km);
+    V w[6][NP], acc[NP], e, v;
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+#pragma unroll
+        for (int q = 0; q < NP; ++q) state_evw<T, ZS>(f, x0[c][q], y0[ZS ? 0 : c][q], e, v, w[c][q]);
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            V n, t;
+            state_evw<T, ZS>(f, xm[a][q], ym[a][q], e, v, n);
+            t = P::sub(w[a][q], n);
+            state_evw<T, ZS>(f, xp[a][q], yp[a][q], e, v, n);
+            t = P::sub(P::add(t, n), w[3 + a][q]);
+            acc[q] = a == 0 ? t : P::add(acc[q], t);
+        }
     T wa, wb;
     {
-        V e_, v_, w_;
-        state_evw<T, ZS>(f, P::make(xa, xb), P::make(ya, yb), e_, v_, w_);
+        V w_;
+        state_evw<T, ZS>(f, P::make(xa, xb), P::make(ya, yb), e, v, w_);
         wa = P::get(w_, 0);
-        if constexpr (P::N == 1) state_evw<T, ZS>(f, P::make(xb, xb), P::make(yb, yb), e_, v_, w_);
+        if constexpr (P::N == 1) state_evw<T, ZS>(f, P::make(xb, xb), P::make(yb, yb), e, v, w_);
         wb = P::get(w_, P::N - 1);
     }
-    V t[NP];
-    row_w(2, o, s0, w);
-    G::shift_down(w, wb, n);
-#pragma unroll
-    for (int q = 0; q < NP; ++q) t[q] = P::sub(w[q], n[q]);
-    row_w(5, o, s0, w);
-    G::shift_up(w, wa, n);
+    V lo[NP], hi[NP];
+    G::shift_down(w[2], wb, lo);
+    G::shift_up(w[5], wa, hi);
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
-        t[q] = P::sub(P::add(t[q], n[q]), w[q]);
-        V r = P::add(acc[q], t[q]);
+        const V t = P::sub(P::add(P::sub(w[2][q], lo[q]), hi[q]), w[5][q]);
+        V r = P::add(acc[q], t);
         if constexpr (!fold_h<T>()) r = P::mul(P::set(div_scale<T>()), r);
 #pragma unroll
         for (int i = 0; i < P::N; ++i) d[q * P::N + i] = P::get(r, i);
