@@ -73,10 +73,11 @@ constexpr int kMaxTimedIters = 2048;
 // update-pass variant per precision, from measurements on GB300: register vectors in
 // ticket-ordered chunks. FP32 waits for memory: half the voxels per thread and three blocks per SM
 // (variant 12, 80 registers, no spills) take 1.58 ms per 512^3 pass against 1.79 ms with two blocks (variant 11) and
-// 1.86 ms with one block of 16-byte vectors (variant 0); 0.236 / 0.266 / 0.274 ms at 256^3. FP64 is ALU-bound:
-// 0.751 ms per 128^3 pass with 16-byte vectors, 0.785 ms with one voxel per thread.
+// 1.86 ms with one block of 16-byte vectors (variant 0); 0.236 / 0.266 / 0.274 ms at 256^3. FP64 is ALU-bound and wants
+// its voxels spread over the SMs: one voxel per thread (variant 11) takes 27 us per 32^3 pass against 37 us with
+// 16-byte vectors, 0.631 against 0.649 ms at 128^3.
 constexpr int kDefaultUpdateVariantF32 = 12;
-constexpr int kDefaultUpdateVariantF64 = 0;
+constexpr int kDefaultUpdateVariantF64 = 11;
 // the captured loop runs the solves of a batch as up to this many independent graph
 // branches, so that one branch's FFT pass (on-chip work) overlaps another branch's
 // streaming passes (HBM work)
@@ -251,21 +252,26 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     if (r.radix_mode > 2) return CCMF_ERR_UNSUPPORTED_SIZE;
     // FFT passes: lines per block (powers of two), shared memory = twiddles + 2 tiles
     auto smem_lines = [&](int n, int L) { return ((size_t)n + 2 * (size_t)n * (L + 1)) * cs; };
-    auto lines_for = [&](int n) {
+    // lines (of `total` per solve) per tile: as many as two tiles in 96 KB allow, at most 16, but few enough that the
+    // tiles of the batch are more than the SMs (kMinTiles): 32 line pairs per block leave a 32^3 solve 32 blocks
+    auto lines_for = [&](int n, long long total) {
         long long L = ((long long)(kSmemBudget / cs) - n) / (2LL * n) - 1;
-        return pow2_floor(L, 16);
+        return fill_tiles(pow2_floor(L, 16), total, batch);
     };
-    auto pick = [&](int want, int n, int* L) {
+    auto pick = [&](int want, int n, long long total, int* L) {
         if (want < 0) {
-            *L = lines_for(n);
+            *L = lines_for(n, total);
             return true;
         }
         if (!pow2_in(want, 1, 16) || smem_lines(n, want) > kSmemMax) return false;
         *L = want;
         return true;
     };
-    if (!pick(r.z_pairs_per_block, n3, &sh.pairs_per_block) || !pick(r.y_lines_per_block, n2, &sh.lpb_y) ||
-        !pick(r.x_lines_per_block, n1, &sh.lpb_x) || !pick(r.zinv_pairs_per_block, n3, &sh.pairs_inv))
+    const long long pairs = ceil_div((long long)n1 * n2, 2), ylines = (long long)pl->n3h * n1,
+                    xlines = (long long)pl->n3h * n2;
+    if (!pick(r.z_pairs_per_block, n3, pairs, &sh.pairs_per_block) ||
+        !pick(r.y_lines_per_block, n2, ylines, &sh.lpb_y) || !pick(r.x_lines_per_block, n1, xlines, &sh.lpb_x) ||
+        !pick(r.zinv_pairs_per_block, n3, pairs, &sh.pairs_inv))
         return CCMF_ERR_UNSUPPORTED_SIZE;
     sh.smem_z = smem_lines(n3, sh.pairs_per_block);
     sh.smem_zi = smem_lines(n3, sh.pairs_inv);
@@ -416,10 +422,9 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     if (explicit_variant && sh.upd_variant != variant) return CCMF_ERR_UNSUPPORTED_SIZE;
     r.update_variant = sh.upd_variant;
     {
-        const int kind = n3 % W != 0 ? kUpdStrided
-                         : sh.upd_variant == 11 ? kUpdHalf2
-                         : sh.upd_variant == 12 ? kUpdHalf3
-                                                : kUpdFull;
+        const int kind = sh.upd_variant == 11 || sh.upd_variant == 12
+                             ? (n3 % 2 != 0 ? kUpdStrided : sh.upd_variant == 11 ? kUpdHalf2 : kUpdHalf3)
+                             : (n3 % W != 0 ? kUpdStrided : kUpdFull);
         const int okind = n3 % W != 0 ? kUpdStrided : kUpdFull;
         sh.upd_resident = (f64 ? update_blocks_per_sm<double>(kind, false) : update_blocks_per_sm<float>(kind, false)) * sms;
         sh.out_resident = (f64 ? update_blocks_per_sm<double>(okind, true) : update_blocks_per_sm<float>(okind, true)) * sms;
@@ -453,7 +458,9 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
         else if (envc && atoi(envc) > 0)
             pb = atoi(envc);
         else
-            pb = one_fits ? 1 : 0;
+            // FP64: one block per plane is bound by its SM's arithmetic, so the line passes win unless the planes
+            // fill the SMs twice (80^3: 41 planes take 192 us, the three line passes 86 us)
+            pb = one_fits && (!f64 || (long long)pl->n3h * batch >= 2 * sms) ? 1 : 0;
     }
     if (pb == 1) {
         if (!one_fits) return CCMF_ERR_UNSUPPORTED_SIZE;
@@ -525,10 +532,11 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     // block tiles on GB300)
     int ze = r.z_engine;
     if (ze < 0) {
-        // measured on GB300: the warp divergence pass wins at N3 = 512 (1.30 against 1.41 ms
-        // per 512^3 pass) and loses at 128; the warp inverse pass wins at both
+        // measured on GB300 (divergence pass, block tiles against one warp per pair): 512^3 1.28 / 0.89 ms,
+        // 256^3 0.188 / 0.129 ms, 128^3 x 3 0.058 / 0.061 ms; 128^3 FP64 0.183 / 0.160 ms. The warp inverse pass wins
+        // at all of them.
         const char* env = getenv("CCMF_Z_ENGINE");
-        const int zdef = n3 >= 512 ? 2 : 1;
+        const int zdef = n3 >= (f64 ? 128 : 256) ? 2 : 1;
         ze = env ? atoi(env) : zdef;
         if (ze < 0 || ze > 2) ze = zdef;
     }
@@ -667,8 +675,9 @@ Ctx<T> make_ctx(const ccmf_plan* pl, unsigned char* ws, const T* gamma, long lon
     c.p.flow = nullptr;
     c.p.run_all = 0;
     const int W = 16 / (int)sizeof(T);
-    c.vec_div = (pl->n3 % W) == 0;
-    c.vec_update = c.vec_div && ((uintptr_t)gamma % 16) == 0;
+    c.vec_div = (pl->n3 % kDivW) == 0;
+    c.vec_update = (pl->n3 % W) == 0 && ((uintptr_t)gamma % 16) == 0;
+    c.pair_update = c.vec_div && ((uintptr_t)gamma % (2 * sizeof(T))) == 0;
     c.p.ab = reinterpret_cast<T*>(ws + pl->off_ab);
     // the stored-divergence schedule needs the vector loads of gamma (a per-solve pointer
     // table is aligned by the batch API's allocations of whole fields)
@@ -1570,7 +1579,7 @@ int batch_persist_capture(ccmf_batch* bt, const std::vector<Ctx<T>>& ctx, unsign
         G.sym_z = c.sym[2];
         G.div_l = make_fastdiv((unsigned)L);
         G.inv_n = (T)(poisson_scale<T>() / (double)c.g.N);
-        G.vec_div = c.vec_div ? 1 : 0;
+        G.vec_div = pl->n3 % (16 / (int)sizeof(T)) == 0 ? 1 : 0;
         G.upd_w = (sizeof(T) == 4 && aligned && pl->n3 % 2 == 0) ? 2 : 1;
         G.nchunks = persist_chunks(c.g.N, G.upd_w);
         const long long pairs = ceil_div((long long)pl->n1 * pl->n2, 2);
@@ -1702,7 +1711,8 @@ int batch_solve_impl(ccmf_batch* bt, const void* const* gammas, const double* xi
         if (bt->persistent) set_state_format(&ctx[b], false);   // k_batch_persist keeps (e, v)
     }
     for (int b = 0; b < nb; ++b) {
-        ctx[b].vec_update = ctx[b].vec_div && aligned;
+        ctx[b].vec_update = bt->plans[b]->n3 % (16 / (int)sizeof(T)) == 0 && aligned;
+        ctx[b].pair_update = ctx[b].vec_div && aligned;
         launch_init<T>(ctx[b], st);
     }
     if (cudaGetLastError() != cudaSuccess) return CCMF_ERR_CUDA;
@@ -1808,7 +1818,8 @@ int batch_time_bucket(ccmf_batch* bt, int b, unsigned char* ws, bool aligned, in
     cfg.resume = 1;
     Ctx<T> c = make_ctx<T>(pl, wsb, nullptr, 0, cfg);
     c.p.gptrs = reinterpret_cast<const T* const*>(ws + bt->gp_off[b]);
-    c.vec_update = c.vec_div && aligned;
+    c.vec_update = pl->n3 % (16 / (int)sizeof(T)) == 0 && aligned;
+    c.pair_update = c.vec_div && aligned;
     if (cudaMemsetAsync(wsb + pl->off_nact, 0, sizeof(int), st) != cudaSuccess) return CCMF_ERR_CUDA;
     launch_init<T>(c, st);   // resume: re-activates the solves without touching their state
     cudaGraph_t graph;

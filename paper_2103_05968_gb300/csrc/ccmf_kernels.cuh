@@ -11,13 +11,13 @@
 //                       (the (div^- grad^+)^+ of Eq. 28), inverse FFT along x;
 //   4. k_fft_lines<2>   inverse FFT along y;
 //   5. k_irfft_z        complex-to-real inverse FFT along z -> phi;
-//   6. k_update<false>  xi^{k+1/2} = w - A(A* w - grad^+ phi - xi_bar) (= P_K(w),
+//   6. k_update         xi^{k+1/2} = w - A(A* w - grad^+ phi - xi_bar) (= P_K(w),
 //                       Eq. 28), over-relaxation, z = v + rho xi, node-wise
 //                       projection onto C_gamma (Eq. 19), e^{k+1}, v^{k+1}
 //                       (Eq. 30), block partial sums; the last block reduces
 //                       them in double and updates rho, the history and the stop
 //                       flag on the device (Eq. 31, BB / LTD scaling).
-// k_update<true> is the final evaluation: it writes the cut xi^{K+1/2} and the
+// (ccmf_update.cuh.) Its OUT instantiation is the final evaluation: it writes the cut xi^{K+1/2} and the
 // flow A* v^K instead of advancing the state.
 #pragma once
 
@@ -1162,12 +1162,11 @@ struct StepConsts {
 // the stencil needs: e/v of w2_a at p + e_a and of w1_a at p - e_a.
 // RULE selects which penalty sums are accumulated (0 BB, 1 constant, 2 LTD,
 // -1 all of them).
-template <typename T, bool OUT, int RULE = -1>
+template <typename T, int RULE = -1>
 __device__ __forceinline__ void voxel_step(const StepConsts<T>& K, const T (&ec)[6], const T (&vc)[6], T gm, T ph0,
                                            const T (&php)[3], const T (&phm)[3], const T (&e2p)[3],
                                            const T (&v2p)[3], const T (&e1m)[3], const T (&v1m)[3],
-                                           T (&acc)[kNSum], T (&eo)[6], T (&vo)[6], T (&flow)[3],
-                                           T* zo = nullptr, bool count = true) {
+                                           T (&acc)[kNSum], T (&eo)[6], T (&vo)[6], bool count = true) {
     T w[6], xh[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) w[c] = ec[c] - vc[c] * K.irho;
@@ -1199,49 +1198,38 @@ __device__ __forceinline__ void voxel_step(const StepConsts<T>& K, const T (&ec)
         acc[kSumRes] += r2;
         acc[kSumPrimal] += gm * Proj<T>::norm(nx2);
     }
-    if (OUT) {
+    T z[6];
+    T nz2 = T(0);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) eo[c] = xh[c];                   // the cut xi^{K+1/2}
+    for (int c = 0; c < 6; ++c) {
+        z[c] = vc[c] + K.rho * (K.alpha * xh[c] - K.beta * ec[c]);
+        nz2 += z[c] * z[c];
+    }
+    const T scale = Proj<T>::scale(nz2, gm);
+    T dvde = T(0), dede = T(0), dvdv = T(0), vv = T(0), ee = T(0);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) flow[a] = K.h * (vc[a] + v2p[a]);  // A* v
-    } else {
-        T z[6];
-        T nz2 = T(0);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            z[c] = vc[c] + K.rho * (K.alpha * xh[c] - K.beta * ec[c]);
-            nz2 += z[c] * z[c];
+    for (int c = 0; c < 6; ++c) {
+        const T vn = z[c] * scale;
+        const T en = (z[c] - vn) * K.irho;
+        if (RULE == 0 || RULE == -1) {
+            const T dv = vn - vc[c], de = en - ec[c];
+            dvde += dv * de;
+            dede += de * de;
+            dvdv += dv * dv;
         }
-        if (zo) {
-#pragma unroll
-            for (int c = 0; c < 6; ++c) zo[c] = z[c];
+        if (RULE == 2 || RULE == -1) {
+            vv += vn * vn;
+            ee += en * en;
         }
-        const T scale = Proj<T>::scale(nz2, gm);
-        T dvde = T(0), dede = T(0), dvdv = T(0), vv = T(0), ee = T(0);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            const T vn = z[c] * scale;
-            const T en = (z[c] - vn) * K.irho;
-            if (RULE == 0 || RULE == -1) {
-                const T dv = vn - vc[c], de = en - ec[c];
-                dvde += dv * de;
-                dede += de * de;
-                dvdv += dv * dv;
-            }
-            if (RULE == 2 || RULE == -1) {
-                vv += vn * vn;
-                ee += en * en;
-            }
-            eo[c] = en;
-            vo[c] = vn;
-        }
-        if (count) {
-            acc[kSumDvDe] += dvde;
-            acc[kSumDeDe] += dede;
-            acc[kSumDvDv] += dvdv;
-            acc[kSumVV] += vv;
-            acc[kSumEE] += ee;
-        }
+        eo[c] = en;
+        vo[c] = vn;
+    }
+    if (count) {
+        acc[kSumDvDe] += dvde;
+        acc[kSumDeDe] += dede;
+        acc[kSumDvDv] += dvdv;
+        acc[kSumVV] += vv;
+        acc[kSumEE] += ee;
     }
 }
 
@@ -1523,9 +1511,9 @@ __global__ void __launch_bounds__(AbVariant<T, VAR>::NW * 32, AbVariant<T, VAR>:
                     const T v2p[3] = {v2x[u], v2y[u], last ? v2z_after : vc[5][(u + 1) % VW]};
                     const T e1m[3] = {e1x[u], e1y[u], first ? e1z_before : ec[2][(u + VW - 1) % VW]};
                     const T v1m[3] = {v1x[u], v1y[u], first ? v1z_before : vc[2][(u + VW - 1) % VW]};
-                    T eou[6], vou[6], fl[3];
-                    voxel_step<T, false>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou, fl,
-                                         nullptr, count);
+                    T eou[6], vou[6];
+                    voxel_step<T>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou,
+                                         count);
 #pragma unroll
                     for (int c = 0; c < 6; ++c) {
                         eo[c][u] = eou[c];
@@ -1668,9 +1656,9 @@ __device__ __forceinline__ void abw_halo_voxel(const StepConsts<T>& K, const T* 
     const T v2p[3] = {__ldg(v + 3 * N + rxp + kh), __ldg(v + 4 * N + ryp + kh), __ldg(v + 5 * N + row + kp)};
     const T e1m[3] = {__ldg(e + 0 * N + rxm + kh), __ldg(e + 1 * N + rym + kh), __ldg(e + 2 * N + row + km)};
     const T v1m[3] = {__ldg(v + 0 * N + rxm + kh), __ldg(v + 1 * N + rym + kh), __ldg(v + 2 * N + row + km)};
-    T acc[kNSum], fl[3];
-    voxel_step<T, false>(K, ec, vc, __ldg(gam + row + kh), __ldg(phi + row + kh), php, phm, e2p, v2p, e1m, v1m,
-                         acc, eo, vo, fl, nullptr, false);
+    T acc[kNSum];
+    voxel_step<T>(K, ec, vc, __ldg(gam + row + kh), __ldg(phi + row + kh), php, phm, e2p, v2p, e1m, v1m,
+                         acc, eo, vo, false);
 }
 
 template <typename T, int VW, int MINB>
@@ -1780,9 +1768,9 @@ __global__ void __launch_bounds__(kAbwWarps * 32, MINB) k_update_abw(Geom g, Ptr
                         const T v2p[3] = {v2x[u], v2y[u], last ? v2z_after : vc[5][(u + 1) % VW]};
                         const T e1m[3] = {e1x[u], e1y[u], first ? e1z_before : ec[2][(u + VW - 1) % VW]};
                         const T v1m[3] = {v1x[u], v1y[u], first ? v1z_before : vc[2][(u + VW - 1) % VW]};
-                        T eou[6], vou[6], fl[3];
-                        voxel_step<T, false>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou,
-                                             fl, nullptr, count);
+                        T eou[6], vou[6];
+                        voxel_step<T>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou,
+                                         count);
 #pragma unroll
                         for (int c = 0; c < 6; ++c) {
                             eo[c][u] = eou[c];
@@ -2129,9 +2117,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_update_tma(Geom g, Ptrs<T> p, L
                 const T v2p[3] = {v2x[u], v2y[u], last ? v2z_after : vc[5][(u + 1) % W]};
                 const T e1m[3] = {e1x[u], e1y[u], first ? e1z_before : ec[2][(u + W - 1) % W]};
                 const T v1m[3] = {v1x[u], v1y[u], first ? v1z_before : vc[2][(u + W - 1) % W]};
-                T eou[6], vou[6], fl[3];
-                voxel_step<T, false, RULE>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou,
-                                           fl);
+                T eou[6], vou[6];
+                voxel_step<T, RULE>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou);
 #pragma unroll
                 for (int c = 0; c < 6; ++c) {
                     eo[c][u] = eou[c];
@@ -2380,8 +2367,8 @@ __global__ void __launch_bounds__(NT) k_update_pipe(Geom g, Ptrs<T> p, LoopConfi
             const T v2p[3] = {v2x[u], v2y[u], last ? v2z_after : vc[5][(u + 1) % W]};
             const T e1m[3] = {e1x[u], e1y[u], first ? e1z_before : ec[2][(u + W - 1) % W]};
             const T v1m[3] = {v1x[u], v1y[u], first ? v1z_before : vc[2][(u + W - 1) % W]};
-            T eou[6], vou[6], fl[3];
-            voxel_step<T, false, RULE>(K, ecu, vcu, gm[u], ph_[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou, fl);
+            T eou[6], vou[6];
+            voxel_step<T, RULE>(K, ecu, vcu, gm[u], ph_[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou);
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
                 eo[c][u] = eou[c];

@@ -30,8 +30,9 @@ struct Ctx {
     const T* rsym[2];     // the x and y tables in digit-reversed order (fused plane pass)
     const double* xi_stage;  // [batch][3] unit normals (device)
     LaunchShape sh;
-    bool vec_div;         // 16-byte path of the divergence pass (N3 % W == 0)
-    bool vec_update;      // 16-byte path of the update pass (also needs gamma 16-byte aligned)
+    bool vec_div;         // pairs of voxels in the divergence pass (N3 even)
+    bool vec_update;      // 16-byte path of the update pass (N3 % W == 0, gamma 16-byte aligned)
+    bool pair_update;     // pairs of voxels in the update pass (N3 even, gamma aligned to a pair)
     bool use_zs;          // the update pass writes the (z, s) state (p.zs is the device's copy)
     bool use_ab;          // stored-divergence schedule: update variants 8 .. 10 write a, b; the first pass reads them
 };
@@ -76,6 +77,16 @@ __global__ void k_setup(SolveScalars* sc, const double* __restrict__ xi, int bat
 }
 
 inline long long ceil_div(long long a, long long b) { return (a + b - 1) / b; }
+
+// Lines per tile of a pass over `total` lines per solve, from the largest that fits: halved while the tiles of all
+// solves are fewer than kMinTiles, about one and a half per SM. Measured (divergence pass): 32^3 FP64 18.5 us with
+// 16 line pairs per block (32 blocks), 12.7 us with 2 (256 blocks), 13.5 us with 1; 64^3 FP32 12.3 us with 16 (128), 10.3
+// us with 8 (256), 12.6 us with 4 (512).
+constexpr long long kMinTiles = 240;
+inline int fill_tiles(int lines, long long total, long long batch) {
+    while (lines > 1 && ceil_div(total, lines) * batch < kMinTiles) lines /= 2;
+    return lines;
+}
 
 // Runs the statement list with the compile-time constant LN equal to the runtime
 // line count L (a power of two <= 16).
@@ -198,7 +209,7 @@ const void* update_kernel(int kind) {
             case kUpdHalf2: return (const void*)k_update<T, WH, false, RULE, F, 2>;
             case kUpdHalf3: return (const void*)k_update<T, WH, false, RULE, F, 3>;
             case kUpdStrided: return (const void*)k_update<T, 0, false, RULE, F, 2>;
-            default: return (const void*)k_update<T, 0, false, -1, false, 2>;
+            default: return (const void*)k_update<T, 0, false, F ? -1 : RULE, false, 2>;
         }
     }
 }
@@ -213,7 +224,7 @@ constexpr int update_voxels(int kind) {
 template <typename T>
 int update_blocks_per_sm(int kind, bool out) {
     int a = 0;
-    const void* f = out ? update_kernel<T, true, -1>(kind) : update_kernel<T, false, -1>(kind);
+    const void* f = out ? update_kernel<T, true, -1>(kind) : update_kernel<T, false, 0>(kind);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, f, kThreads, 0) != cudaSuccess) {
         cudaGetLastError();
         return 1;
@@ -225,8 +236,9 @@ int update_blocks_per_sm(int kind, bool out) {
 template <typename T>
 int update_kind(const Ctx<T>& c) {
     if (sizeof(T) == 4 && !c.use_zs) return kUpdStridedEv;
-    if (!c.vec_update) return kUpdStrided;
-    return c.sh.upd_variant == 11 ? kUpdHalf2 : c.sh.upd_variant == 12 ? kUpdHalf3 : kUpdFull;
+    if (c.sh.upd_variant == 11 || c.sh.upd_variant == 12)
+        return !c.pair_update ? kUpdStrided : c.sh.upd_variant == 11 ? kUpdHalf2 : kUpdHalf3;
+    return c.vec_update ? kUpdFull : kUpdStrided;
 }
 
 #define CCMF_DISPATCH_ABW(var, ...)                                                      \
@@ -578,9 +590,15 @@ void launch_passes(const Ctx<T>& c, const Ptrs<T>& p, cudaStream_t st, F&& betwe
     }
     else {
         const int kind = update_kind(c);
-        const bool bb = c.cfg.rho_rule == 0 || c.cfg.rho_rule == 3;   // the other rules' sums are not needed
-        cudaLaunchKernel(bb ? update_kernel<T, false, 0>(kind) : update_kernel<T, false, -1>(kind),
-                         grid_upd(sh.upd_resident, kind), dim3(kThreads), uargs, 0, st);
+        const int rule = c.cfg.rho_rule;
+        const void* f = nullptr;
+        if (!c.cfg.rho_sched && (rule == 0 || rule == 3))
+            f = update_kernel<T, false, 0>(kind);
+        else if constexpr (sizeof(T) == 4)
+            f = update_kernel<T, false, -1>(kind);
+        else   // FP64 is bound by its arithmetic: no sums that no rule reads
+            f = !c.cfg.rho_sched && rule == 2 ? update_kernel<T, false, 2>(kind) : update_kernel<T, false, 1>(kind);
+        cudaLaunchKernel(f, grid_upd(sh.upd_resident, kind), dim3(kThreads), uargs, 0, st);
     }
     between(kKUpdate);
 }

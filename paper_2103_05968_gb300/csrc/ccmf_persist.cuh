@@ -435,8 +435,8 @@ __device__ void persist_update(const PersistGroup<T>& G, int s, long long ck, co
             const T v2p[3] = {v2x[u], v2y[u], last ? v2z_after : vc[5][(u + 1) % W]};
             const T e1m[3] = {e1x[u], e1y[u], first ? e1z_before : ec[2][(u + W - 1) % W]};
             const T v1m[3] = {v1x[u], v1y[u], first ? v1z_before : vc[2][(u + W - 1) % W]};
-            T eou[6], vou[6], fl[3];
-            voxel_step<T, false>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou, fl);
+            T eou[6], vou[6];
+            voxel_step<T>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou);
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
                 eo[c][u] = eou[c];

@@ -66,6 +66,10 @@ template <> struct VecN<float, 2> {
         const float2 t = __ldg(reinterpret_cast<const float2*>(p));
         o[0] = t.x; o[1] = t.y;
     }
+    __device__ __forceinline__ static void ldcg(const float* p, float (&o)[2]) {
+        const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
+        o[0] = t.x; o[1] = t.y;
+    }
     __device__ __forceinline__ static void st(float* p, const float (&o)[2]) {
         *reinterpret_cast<float2*>(p) = make_float2(o[0], o[1]);
     }
@@ -122,7 +126,14 @@ __device__ __forceinline__ double rsqrt_halley(double x) {
     const double e = fma(-x, y * y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
-__device__ __forceinline__ bool in_float_range(double x) { return x > 1e-30 && x < 1e30; }
+// 2^-100 <= x < 2^100, and a > b for values that are not negative, on the bits (comparisons of doubles occupy the FP64
+// unit too; a NaN compares as larger than anything and passes through the projection as a NaN either way).
+__device__ __forceinline__ bool in_float_range(double x) {
+    return (unsigned)(__double2hiint(x) - (923 << 20)) < (200u << 20);
+}
+__device__ __forceinline__ bool positive_greater(double a, double b) {
+    return __double_as_longlong(a) > __double_as_longlong(b);
+}
 
 // Projection helpers: scale = gamma / |z| when |z| > gamma, else 1, and norm = |x|, from squared norms. FP64
 // compares squares and uses rsqrt_halley where the square lies inside float's range, the IEEE square root and
@@ -132,7 +143,7 @@ template <> struct Proj<double> {
     __device__ __forceinline__ static double scale(double nz2, double gm) {
         double s = 1.0;
         if (in_float_range(nz2)) {
-            if (nz2 > gm * gm) s = gm * rsqrt_halley(nz2);
+            if (positive_greater(nz2, gm * gm)) s = gm * rsqrt_halley(nz2);
         } else {
             const double nz = sqrt(nz2);
             if (nz > gm) s = gm / nz;
@@ -265,16 +276,21 @@ struct Group {
     using Off = GroupOff<T, W>;
     static constexpr int VPT = W > 0 ? W : P::N;   // voxels of the group
     static constexpr int NP = VPT / P::N;          // packs of the group
+    // CG: through L2 only, for data that the same launch writes
+    template <bool CG = false>
     __device__ __forceinline__ static void ld(const T* __restrict__ base, const Off& off, V (&x)[NP]) {
         if constexpr (W > 0) {
             T t[W];
-            VecN<T, W>::ld(base + off.o[0], t);
+            if constexpr (CG)
+                VecN<T, W>::ldcg(base + off.o[0], t);
+            else
+                VecN<T, W>::ld(base + off.o[0], t);
 #pragma unroll
             for (int q = 0; q < NP; ++q) x[q] = P::make(t[q * P::N], t[q * P::N + P::N - 1]);
         } else {
             T t[P::N];
 #pragma unroll
-            for (int i = 0; i < P::N; ++i) t[i] = __ldg(base + off.o[i]);
+            for (int i = 0; i < P::N; ++i) t[i] = CG ? __ldcg(base + off.o[i]) : __ldg(base + off.o[i]);
             x[0] = P::make(t[0], t[P::N - 1]);
         }
     }

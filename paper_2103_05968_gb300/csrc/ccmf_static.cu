@@ -165,9 +165,9 @@ int static_solve(int n1, int n2, int n3, const T* gamma, const double* xi_bar, c
         if (!radix_plan(nn[a], &c.ax[a])) return CCMF_ERR_UNSUPPORTED_SIZE;
     const size_t cs = 2 * sizeof(T);
     LaunchShape& sh = c.sh;
-    sh.pairs_per_block = lines_for(n3, cs);
-    sh.lpb_y = lines_for(n2, cs);
-    sh.lpb_x = lines_for(n1, cs);
+    sh.pairs_per_block = fill_tiles(lines_for(n3, cs), ceil_div((long long)n1 * n2, 2), 1);
+    sh.lpb_y = fill_tiles(lines_for(n2, cs), (long long)g.n3h * n1, 1);
+    sh.lpb_x = fill_tiles(lines_for(n1, cs), (long long)g.n3h * n2, 1);
     sh.smem_z = ((size_t)n3 + 2 * (size_t)n3 * (sh.pairs_per_block + 1)) * cs;
     sh.pairs_inv = sh.pairs_per_block;
     sh.smem_zi = sh.smem_z;
@@ -176,7 +176,7 @@ int static_solve(int n1, int n2, int n3, const T* gamma, const double* xi_bar, c
     long long gu = (g.N + kThreads - 1) / kThreads;
     sh.grid_update = (int)(gu < kStaticGridUpdate ? gu : kStaticGridUpdate);
     sh.upd_resident = sh.out_resident = 0;   // the update pass runs grid_update blocks per solve
-    sh.upd_variant = sizeof(T) == 4 ? 12 : 0;
+    sh.upd_variant = sizeof(T) == 4 ? 12 : 11;
 
     // scratch layout: scalars, counter, normal, partials, history, state (two copies),
     // spectrum, phi, tables
@@ -244,8 +244,9 @@ int static_solve(int n1, int n2, int n3, const T* gamma, const double* xi_bar, c
     c.p.gamma = gamma;
     c.p.gstride = 0;
     const int W = 16 / (int)sizeof(T);
-    c.vec_div = (n3 % W) == 0;
-    c.vec_update = c.vec_div && ((uintptr_t)gamma % 16) == 0;
+    c.vec_div = (n3 % kDivW) == 0;
+    c.vec_update = (n3 % W) == 0 && ((uintptr_t)gamma % 16) == 0;
+    c.pair_update = c.vec_div && ((uintptr_t)gamma % (2 * sizeof(T))) == 0;
     c.use_zs = sizeof(T) == 4;
     c.p.zs = c.use_zs ? 1 : 0;
 

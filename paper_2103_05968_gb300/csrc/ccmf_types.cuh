@@ -25,21 +25,20 @@ constexpr int kHistFields = 6;
 constexpr int kHistCap = 4096;   // history entries reserved per solve
 constexpr int kThreads = 256;
 
-// The register update pass works in chunks, taken in order, with one partial-sum slot per chunk. A chunk is
-// kVecChunkGroups groups per thread (8 K voxels in FP32 with two voxels per group) on large grids. Grids that would give
-// fewer than kVecMinChunks chunks halve it until they do, so that the chunks spread over the SMs: 16 groups
-// give a 32^3 FP64 solve 4 chunks, i.e. 4 busy SMs (436 us a pass). In FP32 400 chunks were the best of 96, 400
-// and 1300 (96^3 x 6: 98 / 88 / 118 us a pass, 128^3 x 3: 194 / 185 / 202 us an iteration); in FP64, where a chunk's
-// arithmetic is long, 1300 (128^3: 735 / 741 / 700 us). The rule depends on the grid and the precision alone, so a
-// solve sums in the same order alone and in a batch.
+// The register update pass works in chunks, taken in order, with one partial-sum slot per chunk. A chunk is at
+// most kVecChunkGroups groups per thread (8 K voxels in FP32 with two voxels per group). With chunks of that size on
+// every grid a 32^3 FP64 solve had 4 chunks, i.e. 4 busy SMs, and 436 us a pass.
+// The size is halved until there are enough chunks: 400 in FP32, 1300 in FP64, where a group's arithmetic is long
+// (128^3 update 735 us with 96, 741 with 400, 700 with 1300).
+// The rule depends on the grid and the precision alone, so a solve sums in the same order alone and in a batch.
 constexpr int kVecChunkGroups = 16;
 template <typename T>
 __host__ __device__ inline int vec_chunk_groups(long long n_voxels, int voxels_per_group) {
-    constexpr long long kVecMinChunks = sizeof(T) == 4 ? 400 : 1300;
+    constexpr int kVecMinChunks = sizeof(T) == 4 ? 400 : 1300;
     const long long per_block = (long long)kThreads * voxels_per_group;
     const long long groups = (n_voxels + per_block - 1) / per_block;
     int per = kVecChunkGroups;
-    while (per > 1 && groups < kVecMinChunks * per) per /= 2;
+    while (per > 1 && groups < (long long)kVecMinChunks * per) per /= 2;
     return per;
 }
 template <typename T>

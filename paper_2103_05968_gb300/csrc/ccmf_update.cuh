@@ -26,11 +26,43 @@ struct UpdIo {
     T* zout;                // z = v + rho xi of an (e, v)-format update, may be null
 };
 
+template <typename T>
+__device__ __forceinline__ UpdConsts<T> upd_consts(const StepConsts<T>& C) {
+    using P = Pk<T>;
+    UpdConsts<T> K;
+    K.h = P::set(C.h);
+    K.nh = P::set(-C.h);
+    K.half = P::set(T(0.5));
+    K.alpha = P::set(C.alpha);
+    K.nbeta = P::set(-C.beta);
+    K.rho = P::set(C.rho);
+    K.irho = P::set(C.irho);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) K.xi[a] = P::set(fold_h<T>() ? C.hxi[a] : C.xi[a]);
+    return K;
+}
+
+template <typename T, bool OUT>
+__device__ __forceinline__ UpdIo<T> upd_io(const Ptrs<T>& p, const SolveScalars& S, int s, long long N,
+                                           const T (&recip)[2]) {
+    const long long other = (long long)(1 - (S.iters & 1)) * p.sstride + (long long)s * 6 * N;
+    UpdIo<T> io;
+    io.f = state_src<T>(p, S, s, N, recip);
+    io.phi = p.phi + (size_t)s * N;
+    io.gam = gamma_of(p, s);
+    io.ao = p.e + other;
+    io.bo = p.v + other;
+    io.cut = OUT && p.cut ? p.cut + (size_t)s * 6 * N : nullptr;
+    io.flow = OUT && p.flow ? p.flow + (size_t)s * 3 * N : nullptr;
+    io.zout = !OUT && p.zout ? p.zout + (size_t)s * 6 * N : nullptr;
+    return io;
+}
+
 // One group of the update. OUT: the final evaluation (cut, flow, sums of the state) instead of an
-// update. RZS / WZS: the format read / written. RULE 0 accumulates the sums of the BB and
-// residual-balancing rules, -1 all of them. mask: 1 per voxel that counts (a strided pack whose second
+// update. RZS / WZS: the format read / written. RULE: the penalty sums accumulated: 0 those of the BB and
+// residual-balancing rules, 1 none (constant or replayed penalties), 2 the LTD rule's, -1 all. mask: 1 per voxel that counts (a strided pack whose second
 // voxel lies beyond the grid repeats the first with mask 0).
-template <typename T, int W, bool OUT, int RULE, bool RZS, bool WZS>
+template <typename T, int W, bool OUT, int RULE, bool RZS, bool WZS, bool CG = false>
 __device__ __forceinline__ void update_group(const Geom& g, const UpdIo<T>& io, const UpdConsts<T>& K, long long lin0,
                                              long long lin1, bool valid, typename Pk<T>::V (&acc)[kNSum]) {
     using P = Pk<T>;
@@ -82,20 +114,21 @@ __device__ __forceinline__ void update_group(const Geom& g, const UpdIo<T>& io, 
     };
     V gm[NP], ph[NP], w2p[3][NP], v2p[3][NP], w1m[3][NP], php[3][NP], phm[3][NP], vdump[NP];
     G::ld(io.gam, own, gm);
-    G::ld(io.phi, own, ph);
+    G::template ld<CG>(io.phi, own, ph);
     other(3, ip, w2p[0], v2p[0]);
     other(0, im, w1m[0], vdump);
     other(4, jp, w2p[1], v2p[1]);
     other(1, jm, w1m[1], vdump);
-    G::ld(io.phi, ip, php[0]);
-    G::ld(io.phi, im, phm[0]);
-    G::ld(io.phi, jp, php[1]);
-    G::ld(io.phi, jm, phm[1]);
+    G::template ld<CG>(io.phi, ip, php[0]);
+    G::template ld<CG>(io.phi, im, phm[0]);
+    G::template ld<CG>(io.phi, jp, php[1]);
+    G::template ld<CG>(io.phi, jm, phm[1]);
     if constexpr (W > 0) {
         // z neighbours: inside the group, or one voxel on each side of it
         const T xa = __ldg(f.a + 5 * N + kp.o[0]), ya = __ldg((RZS ? f.b : f.b + 5 * N) + kp.o[0]);
         const T xb = __ldg(f.a + 2 * N + km.o[0]), yb = __ldg((RZS ? f.b : f.b + 2 * N) + km.o[0]);
-        const T pa = __ldg(io.phi + kp.o[0]), pb = __ldg(io.phi + km.o[0]);
+        const T pa = CG ? __ldcg(io.phi + kp.o[0]) : __ldg(io.phi + kp.o[0]);
+        const T pb = CG ? __ldcg(io.phi + km.o[0]) : __ldg(io.phi + km.o[0]);
         T wa, wb, va;
         V e_, v_, w_;
         if constexpr (P::N == 2) {
@@ -118,11 +151,19 @@ __device__ __forceinline__ void update_group(const Geom& g, const UpdIo<T>& io, 
     } else {
         other(5, kp, w2p[2], v2p[2]);
         other(2, km, w1m[2], vdump);
-        G::ld(io.phi, kp, php[2]);
-        G::ld(io.phi, km, phm[2]);
+        G::template ld<CG>(io.phi, kp, php[2]);
+        G::template ld<CG>(io.phi, km, phm[2]);
     }
     const V mask = P::make(T(1), valid ? T(1) : T(0));
     auto take = [&](int i, V x) { acc[i] = (W > 0 || P::N == 1) ? P::add(acc[i], x) : P::fma(x, mask, acc[i]); };
+    // FP64 sums products straight into the accumulators (one addition less per sum); FP32 sums a voxel's six first
+    constexpr bool kDirect = sizeof(T) == 8;
+    auto sum_sq = [&](int i, V a, V b, V& local) {
+        if constexpr (kDirect)
+            acc[i] = P::fma(a, b, acc[i]);
+        else
+            local = P::fma(a, b, local);
+    };
     V oa[6][NP], ob[6][NP], of[3][NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
@@ -147,7 +188,7 @@ __device__ __forceinline__ void update_group(const Geom& g, const UpdIo<T>& io, 
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             const V d = P::sub(x[c], ec[c][q]);
-            r2 = P::fma(d, d, r2);
+            sum_sq(kSumRes, d, d, r2);
             nx2 = P::fma(x[c], x[c], nx2);
             take(kSumV + c, vc[c][q]);
             if constexpr (OUT) {
@@ -160,8 +201,11 @@ __device__ __forceinline__ void update_group(const Geom& g, const UpdIo<T>& io, 
                 nz2 = P::fma(z[c], z[c], nz2);
             }
         }
-        take(kSumRes, r2);
-        take(kSumPrimal, P::mul(gm[q], P::norm(nx2)));
+        if constexpr (!kDirect) take(kSumRes, r2);
+        if constexpr (kDirect)
+            acc[kSumPrimal] = P::fma(gm[q], P::norm(nx2), acc[kSumPrimal]);
+        else
+            take(kSumPrimal, P::mul(gm[q], P::norm(nx2)));
         if constexpr (!OUT) {
             const V s = P::scale(nz2, gm[q]);
             const V te = P::mul(P::sub(P::set(T(1)), s), K.irho);
@@ -172,12 +216,14 @@ __device__ __forceinline__ void update_group(const Geom& g, const UpdIo<T>& io, 
                 // e' = (z - v') / rho; FP64 saves an operation a component by z ((1 - s) / rho)
                 const V en = fold_h<T>() ? P::mul(z[c], te) : P::mul(P::sub(z[c], vn), K.irho);
                 const V dv = P::sub(vn, vc[c][q]), de = P::sub(en, ec[c][q]);
-                dvde = P::fma(dv, de, dvde);
-                dede = P::fma(de, de, dede);
-                dvdv = P::fma(dv, dv, dvdv);
-                if constexpr (RULE == -1) {
-                    vv = P::fma(vn, vn, vv);
-                    ee = P::fma(en, en, ee);
+                if constexpr (RULE == 0 || RULE == -1) {
+                    sum_sq(kSumDvDe, dv, de, dvde);
+                    sum_sq(kSumDeDe, de, de, dede);
+                    sum_sq(kSumDvDv, dv, dv, dvdv);
+                }
+                if constexpr (RULE == 2 || RULE == -1) {
+                    sum_sq(kSumVV, vn, vn, vv);
+                    sum_sq(kSumEE, en, en, ee);
                 }
                 if constexpr (WZS) {
                     oa[c][q] = z[c];
@@ -187,10 +233,12 @@ __device__ __forceinline__ void update_group(const Geom& g, const UpdIo<T>& io, 
                 }
             }
             if constexpr (WZS) ob[0][q] = s;
-            take(kSumDvDe, dvde);
-            take(kSumDeDe, dede);
-            take(kSumDvDv, dvdv);
-            if constexpr (RULE == -1) {
+            if constexpr (!kDirect && (RULE == 0 || RULE == -1)) {
+                take(kSumDvDe, dvde);
+                take(kSumDeDe, dede);
+                take(kSumDvDv, dvdv);
+            }
+            if constexpr (!kDirect && (RULE == 2 || RULE == -1)) {
                 take(kSumVV, vv);
                 take(kSumEE, ee);
             }
@@ -264,27 +312,8 @@ __global__ void __launch_bounds__(kThreads, MINB) k_update(Geom g, Ptrs<T> p, Lo
         state_recip<T>(S, recip);
     }
     __syncthreads();
-    UpdConsts<T> K;
-    K.h = P::set(C.h);
-    K.nh = P::set(-C.h);
-    K.half = P::set(T(0.5));
-    K.alpha = P::set(C.alpha);
-    K.nbeta = P::set(-C.beta);
-    K.rho = P::set(C.rho);
-    K.irho = P::set(C.irho);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) K.xi[a] = P::set(fold_h<T>() ? C.hxi[a] : C.xi[a]);
-    const int par = S.iters & 1;
-    const long long other = (long long)(1 - par) * p.sstride + (long long)s * 6 * N;
-    UpdIo<T> io;
-    io.f = state_src<T>(p, S, s, N, recip);
-    io.phi = p.phi + (size_t)s * N;
-    io.gam = gamma_of(p, s);
-    io.ao = p.e + other;
-    io.bo = p.v + other;
-    io.cut = OUT && p.cut ? p.cut + (size_t)s * 6 * N : nullptr;
-    io.flow = OUT && p.flow ? p.flow + (size_t)s * 3 * N : nullptr;
-    io.zout = !OUT && p.zout ? p.zout + (size_t)s * 6 * N : nullptr;
+    const UpdConsts<T> K = upd_consts<T>(C);
+    const UpdIo<T> io = upd_io<T, OUT>(p, S, s, N, recip);
     const bool rzs = state_is_zs<T>(S);
     const int cgroups = vec_chunk_groups<T>(N, VPT);
     double* part = p.partial + (size_t)s * nchunks * kNSum;
