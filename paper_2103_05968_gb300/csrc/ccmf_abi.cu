@@ -1579,9 +1579,9 @@ int batch_persist_capture(ccmf_batch* bt, const std::vector<Ctx<T>>& ctx, unsign
         G.sym_z = c.sym[2];
         G.div_l = make_fastdiv((unsigned)L);
         G.inv_n = (T)(poisson_scale<T>() / (double)c.g.N);
-        G.vec_div = pl->n3 % (16 / (int)sizeof(T)) == 0 ? 1 : 0;
+        G.vec_div = c.vec_div ? 1 : 0;
         G.upd_w = (sizeof(T) == 4 && aligned && pl->n3 % 2 == 0) ? 2 : 1;
-        G.nchunks = persist_chunks(c.g.N, G.upd_w);
+        G.nchunks = persist_chunks(c.g.N, sizeof(T) == 4 ? 2 : 1);
         const long long pairs = ceil_div((long long)pl->n1 * pl->n2, 2);
         G.tiles[0] = (int)ceil_div(pairs, P);
         G.tiles[1] = (int)ceil_div((long long)pl->n3h * pl->n1, L);
@@ -1708,7 +1708,7 @@ int batch_solve_impl(ccmf_batch* bt, const void* const* gammas, const double* xi
             return CCMF_ERR_CUDA;
         ctx[b] = make_ctx<T>(pl, wsb, nullptr, 0, cfg);
         ctx[b].p.gptrs = reinterpret_cast<const T* const*>(ws + bt->gp_off[b]);
-        if (bt->persistent) set_state_format(&ctx[b], false);   // k_batch_persist keeps (e, v)
+        set_state_format(&ctx[b], bt->persistent ? sizeof(T) == 4 : ctx[b].use_zs);   // the format k_batch_persist runs
     }
     for (int b = 0; b < nb; ++b) {
         ctx[b].vec_update = bt->plans[b]->n3 % (16 / (int)sizeof(T)) == 0 && aligned;

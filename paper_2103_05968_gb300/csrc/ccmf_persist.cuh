@@ -29,7 +29,7 @@
 // path as in the other kernels.
 #pragma once
 
-#include "ccmf_kernels.cuh"
+#include "ccmf_update.cuh"
 
 namespace ccmf {
 
@@ -54,8 +54,8 @@ struct PersistGroup {
     const T* sym_z;             // 4 sin^2(pi k / n3), natural order
     FastDiv div_l;              // the tile's line count L (in-place stage indexing)
     T inv_n;                    // poisson_scale / N
-    int vec_div;                // pass 0 reads 16-byte vectors (n3 % (16 / sizeof(T)) == 0)
-    int upd_w;                  // voxels per thread group of pass 5 (vector width)
+    int vec_div;                // pass 0 reads pairs of voxels (n3 even)
+    int upd_w;                  // 2: pass 5 runs on vectors of two voxels (FP32), 1: on strided packs
     long long nchunks;          // pass-5 chunks per solve
     int tiles[kPersistPasses];  // tiles per solve of each pass (pass 5: chunks)
     int tpi[kPersistPasses];    // consecutive tiles per work item (1 for pass 5: one partial slot per chunk)
@@ -83,21 +83,6 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
 
 __device__ __forceinline__ float2 ldcg_cx(const float2* p) { return __ldcg(p); }
 __device__ __forceinline__ double2 ldcg_cx(const double2* p) { return __ldcg(p); }
-
-// W consecutive elements through L2 only.
-template <typename T, int W> struct VecCg;
-template <> struct VecCg<float, 2> {
-    __device__ __forceinline__ static void ld(const float* p, float (&o)[2]) {
-        const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
-        o[0] = t.x; o[1] = t.y;
-    }
-};
-template <> struct VecCg<float, 1> {
-    __device__ __forceinline__ static void ld(const float* p, float (&o)[1]) { o[0] = __ldcg(p); }
-};
-template <> struct VecCg<double, 1> {
-    __device__ __forceinline__ static void ld(const double* p, double (&o)[1]) { o[0] = __ldcg(p); }
-};
 
 // Dynamic shared memory of k_batch_persist, in three parts: the queue tables (first item of
 // every (pass, group), each group's scalar slots, first solve and tiles per pass), the
@@ -128,24 +113,22 @@ __device__ void persist_div_rfft_z(const PersistGroup<T>& G, int s, long long t,
                                    unsigned char* work) {
     using C = cx<T>;
     constexpr int stride = P + 1;
-    constexpr int W = VEC ? Vec16<T>::W : 1;
+    constexpr int W = VEC ? kDivW : 1;
+    constexpr bool ZS = sizeof(T) == 4;   // the state format of the persistent launch
     const Geom& g = G.g;
     const Ptrs<T>& p = G.p;
     C* A = reinterpret_cast<C*>(work);
     C* B = A + (size_t)g.n3 * stride;
-    const T irho = T(1) / (T)p.sc[s].rho;
-    const long long N = g.N;
-    const long long cur = (long long)(p.sc[s].iters & 1) * p.sstride + (long long)s * 6 * N;
-    const T* __restrict__ e = p.e + cur;
-    const T* __restrict__ v = p.v + cur;
+    T recip[2];
+    state_recip<T>(p.sc[s], recip);
+    const StateSrc<T> f = state_src<T>(p, p.sc[s], s, g.N, recip);
     const long long Lp = (long long)g.n1 * g.n2;
     const long long l0 = t * 2 * P;
-    const int n3w = g.n3 / W;
-    const int cnt = 2 * P * n3w;
+    const int cnt = 2 * P * g.n3 / W;
     T* Ar = reinterpret_cast<T*>(A);
     for (int idx = threadIdx.x; idx < cnt; idx += kThreads) {
-        const int ll = idx / n3w;
-        const int k0 = (idx - ll * n3w) * W;
+        const int ll = (int)fdiv((unsigned)(idx * W), g.div_n3);
+        const int k0 = idx * W - ll * g.n3;
         const long long l = l0 + ll;
         T d[W];
 #pragma unroll
@@ -154,51 +137,10 @@ __device__ void persist_div_rfft_z(const PersistGroup<T>& G, int s, long long t,
             const RowNb rn = row_neighbours(g, (unsigned)l);
             const int kp = (k0 + W == g.n3) ? 0 : k0 + W;
             const int km = (k0 == 0) ? g.n3 - 1 : k0 - 1;
-            if constexpr (VEC) {
-                T w[6][W], te[W], tv[W];
-#pragma unroll
-                for (int c = 0; c < 6; ++c) {
-                    Vec16<T>::ld(e + c * N + rn.row + k0, te);
-                    Vec16<T>::ld(v + c * N + rn.row + k0, tv);
-#pragma unroll
-                    for (int u = 0; u < W; ++u) w[c][u] = te[u] - tv[u] * irho;
-                }
-                T xp[W], xm[W], yp[W], ym[W];
-                Vec16<T>::ld(e + 3 * N + rn.ip + k0, te);
-                Vec16<T>::ld(v + 3 * N + rn.ip + k0, tv);
-#pragma unroll
-                for (int u = 0; u < W; ++u) xp[u] = te[u] - tv[u] * irho;
-                Vec16<T>::ld(e + 0 * N + rn.im + k0, te);
-                Vec16<T>::ld(v + 0 * N + rn.im + k0, tv);
-#pragma unroll
-                for (int u = 0; u < W; ++u) xm[u] = te[u] - tv[u] * irho;
-                Vec16<T>::ld(e + 4 * N + rn.jp + k0, te);
-                Vec16<T>::ld(v + 4 * N + rn.jp + k0, tv);
-#pragma unroll
-                for (int u = 0; u < W; ++u) yp[u] = te[u] - tv[u] * irho;
-                Vec16<T>::ld(e + 1 * N + rn.jm + k0, te);
-                Vec16<T>::ld(v + 1 * N + rn.jm + k0, tv);
-#pragma unroll
-                for (int u = 0; u < W; ++u) ym[u] = te[u] - tv[u] * irho;
-                const T zp = __ldg(e + 5 * N + rn.row + kp) - __ldg(v + 5 * N + rn.row + kp) * irho;
-                const T zm = __ldg(e + 2 * N + rn.row + km) - __ldg(v + 2 * N + rn.row + km) * irho;
-#pragma unroll
-                for (int u = 0; u < W; ++u) {
-                    const T w2zp = (u + 1 < W) ? w[5][(u + 1) % W] : zp;
-                    const T w1zm = (u > 0) ? w[2][(u + W - 1) % W] : zm;
-                    const T sx = w[0][u] - xm[u] + xp[u] - w[3][u];
-                    const T sy = w[1][u] - ym[u] + yp[u] - w[4][u];
-                    const T sz = w[2][u] - w1zm + w2zp - w[5][u];
-                    d[u] = div_scale<T>() * (sx + sy + sz);
-                }
-            } else {
-                const long long p0 = rn.row + k0;
-                auto wc = [&](int c, long long off) { return e[c * N + off] - v[c * N + off] * irho; };
-                const T sx = wc(0, p0) - wc(0, rn.im + k0) + wc(3, rn.ip + k0) - wc(3, p0);
-                const T sy = wc(1, p0) - wc(1, rn.jm + k0) + wc(4, rn.jp + k0) - wc(4, p0);
-                const T sz = wc(2, p0) - wc(2, rn.row + km) + wc(5, rn.row + kp) - wc(5, p0);
-                d[0] = div_scale<T>() * (sx + sy + sz);
-            }
+            if constexpr (VEC)
+                div_group<T, ZS>(f, rn, k0, kp, km, d);
+            else
+                d[0] = div_voxel<T, ZS>(f, rn, k0, kp, km);
         }
 #pragma unroll
         for (int u = 0; u < W; ++u) Ar[2 * ((k0 + u) * stride + (ll >> 1)) + (ll & 1)] = d[u];
@@ -365,91 +307,34 @@ __host__ __device__ inline long long persist_chunks(long long n_voxels, int voxe
 
 template <typename T, int W>
 __device__ void persist_update(const PersistGroup<T>& G, int s, long long ck, const LoopConfig& cfg) {
-    using V = VecN<T, W>;
-    using VC = VecCg<T, W>;
+    using P = Pk<T>;
+    using V = typename P::V;
+    constexpr bool ZS = sizeof(T) == 4;
+    constexpr int VPT = Group<T, W>::VPT;
     const Geom& g = G.g;
     const Ptrs<T>& p = G.p;
     const SolveScalars& S = p.sc[s];
     const long long N = g.N;
-    const StepConsts<T> K = step_consts<T>(S, cfg);
-    const int par = S.iters & 1;
-    const T* __restrict__ e = p.e + (long long)par * p.sstride + (long long)s * 6 * N;
-    const T* __restrict__ v = p.v + (long long)par * p.sstride + (long long)s * 6 * N;
-    T* __restrict__ e_out = p.e + (long long)(1 - par) * p.sstride + (long long)s * 6 * N;
-    T* __restrict__ v_out = p.v + (long long)(1 - par) * p.sstride + (long long)s * 6 * N;
-    const T* phi = p.phi + (size_t)s * N;   // written by pass 4 of this launch: L2-only loads
-    const T* __restrict__ gam = gamma_of(p, s);
-    const long long ngroups = N / W;
-    T acc[kNSum];
+    const UpdConsts<T> K = upd_consts<T>(step_consts<T>(S, cfg));
+    T recip[2];
+    state_recip<T>(S, recip);
+    const UpdIo<T> io = upd_io<T, false>(p, S, s, N, recip);
+    V acc[kNSum];
 #pragma unroll
-    for (int q = 0; q < kNSum; ++q) acc[q] = T(0);
+    for (int q = 0; q < kNSum; ++q) acc[q] = P::set(T(0));
 #pragma unroll 1
     for (int gi = 0; gi < kPersistChunkGroups; ++gi) {
-        const long long q = (ck * kPersistChunkGroups + gi) * kThreads + threadIdx.x;
-        if (q >= ngroups) break;
-        const long long lin0 = q * W;
-        const unsigned row = fdiv((unsigned)lin0, g.div_n3);
-        const int k0 = (int)(lin0 - (long long)row * g.n3);
-        const RowNb rn = row_neighbours(g, row);
-        const int kp = (k0 + W == g.n3) ? 0 : k0 + W;
-        const int km = (k0 == 0) ? g.n3 - 1 : k0 - 1;
-        T ec[6][W], vc[6][W];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            V::ld(e + c * N + lin0, ec[c]);
-            V::ld(v + c * N + lin0, vc[c]);
-        }
-        T gm[W], ph[W];
-        V::ld(gam + lin0, gm);
-        VC::ld(phi + lin0, ph);
-        T e2x[W], v2x[W], e1x[W], v1x[W], e2y[W], v2y[W], e1y[W], v1y[W];
-        T phxp[W], phxm[W], phyp[W], phym[W];
-        V::ld(e + 3 * N + rn.ip + k0, e2x);
-        V::ld(v + 3 * N + rn.ip + k0, v2x);
-        V::ld(e + 0 * N + rn.im + k0, e1x);
-        V::ld(v + 0 * N + rn.im + k0, v1x);
-        V::ld(e + 4 * N + rn.jp + k0, e2y);
-        V::ld(v + 4 * N + rn.jp + k0, v2y);
-        V::ld(e + 1 * N + rn.jm + k0, e1y);
-        V::ld(v + 1 * N + rn.jm + k0, v1y);
-        VC::ld(phi + rn.ip + k0, phxp);
-        VC::ld(phi + rn.im + k0, phxm);
-        VC::ld(phi + rn.jp + k0, phyp);
-        VC::ld(phi + rn.jm + k0, phym);
-        const T e2z_after = __ldg(e + 5 * N + rn.row + kp), v2z_after = __ldg(v + 5 * N + rn.row + kp);
-        const T e1z_before = __ldg(e + 2 * N + rn.row + km), v1z_before = __ldg(v + 2 * N + rn.row + km);
-        const T ph_after = __ldcg(phi + rn.row + kp), ph_before = __ldcg(phi + rn.row + km);
-        T eo[6][W], vo[6][W];
-#pragma unroll
-        for (int u = 0; u < W; ++u) {
-            T ecu[6], vcu[6];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                ecu[c] = ec[c][u];
-                vcu[c] = vc[c][u];
-            }
-            const bool last = (u + 1 == W), first = (u == 0);
-            const T php[3] = {phxp[u], phyp[u], last ? ph_after : ph[(u + 1) % W]};
-            const T phm[3] = {phxm[u], phym[u], first ? ph_before : ph[(u + W - 1) % W]};
-            const T e2p[3] = {e2x[u], e2y[u], last ? e2z_after : ec[5][(u + 1) % W]};
-            const T v2p[3] = {v2x[u], v2y[u], last ? v2z_after : vc[5][(u + 1) % W]};
-            const T e1m[3] = {e1x[u], e1y[u], first ? e1z_before : ec[2][(u + W - 1) % W]};
-            const T v1m[3] = {v1x[u], v1y[u], first ? v1z_before : vc[2][(u + W - 1) % W]};
-            T eou[6], vou[6];
-            voxel_step<T>(K, ecu, vcu, gm[u], ph[u], php, phm, e2p, v2p, e1m, v1m, acc, eou, vou);
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                eo[c][u] = eou[c];
-                vo[c][u] = vou[c];
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            V::st(e_out + c * N + lin0, eo[c]);
-            V::st(v_out + c * N + lin0, vo[c]);
-        }
+        const long long gb = (ck * kPersistChunkGroups + gi) * kThreads;
+        const long long lin0 = W > 0 ? (gb + threadIdx.x) * W : gb * VPT + threadIdx.x;
+        if (lin0 >= N) break;
+        const bool valid = W > 0 || lin0 + kThreads < N;
+        // phi comes from pass 4 of this launch: L2-only loads
+        update_group<T, W, false, -1, ZS, ZS, true>(g, io, K, lin0, valid ? lin0 + kThreads : lin0, valid, acc);
     }
-    block_store_partial<T, kNSum>(acc, p.partial + (size_t)s * G.nchunks * kNSum, ck);
+    T sums[kNSum];
+#pragma unroll
+    for (int q = 0; q < kNSum; ++q) sums[q] = P::sum(acc[q]);
+    block_store_partial<T, kNSum>(sums, p.partial + (size_t)s * G.nchunks * kNSum, ck);
 }
 
 // Bounded wait of thread 0 until *ctr >= need (acquire). Returns false when the budget
@@ -594,9 +479,9 @@ __global__ void __launch_bounds__(kThreads, kPersistMinBlocks) k_batch_persist(P
                         if (sg.upd_w == 2)
                             persist_update<T, 2>(sg, s, tile, a.cfg);
                         else
-                            persist_update<T, 1>(sg, s, tile, a.cfg);
+                            persist_update<T, 0>(sg, s, tile, a.cfg);
                     } else {
-                        persist_update<T, 1>(sg, s, tile, a.cfg);
+                        persist_update<T, 0>(sg, s, tile, a.cfg);
                     }
                     break;
             }
@@ -614,7 +499,7 @@ __global__ void __launch_bounds__(kThreads, kPersistMinBlocks) k_batch_persist(P
             // the penalty rule, history row and stop test (rho, iters, active change here)
             SolveScalars& S = sg.p.sc[s];
             const double* part = sg.p.partial + (size_t)s * sg.nchunks * kNSum;
-            update_finish<T, false>(sg.g, sg.p, a.cfg, S, s, S.rho, part, (int)sg.nchunks);
+            update_finish<T, false, kThreads, false, sizeof(T) == 4>(sg.g, sg.p, a.cfg, S, s, S.rho, part, (int)sg.nchunks);
         }
     }
 }

@@ -28,15 +28,22 @@ constexpr int kThreads = 256;
 // The register update pass works in chunks, taken in order, with one partial-sum slot per chunk. A chunk is at
 // most kVecChunkGroups groups per thread (8 K voxels in FP32 with two voxels per group). With chunks of that size on
 // every grid a 32^3 FP64 solve had 4 chunks, i.e. 4 busy SMs, and 436 us a pass.
-// The size is halved until there are enough chunks: 400 in FP32, 1300 in FP64, where a group's arithmetic is long
-// (128^3 update 735 us with 96, 741 with 400, 700 with 1300).
+// FP32: where one round of the kVecSlots blocks that are resident on GB300 (three per SM) can take the grid, the
+// chunks are sized for just that round (128^3: 456 chunks of 9 groups, 92 us for three solves; 512 of 8, 103 us);
+// above it they stay whole (256^3: 211 us with 16 groups, 237 us with five rounds of 15, whose ends cut rows).
+// FP64, where a group's arithmetic is long: halved from 16 until there are kVecMinChunks (128^3 update 735 us with
+// 96, 741 with 400, 700 with 1300).
 // The rule depends on the grid and the precision alone, so a solve sums in the same order alone and in a batch.
 constexpr int kVecChunkGroups = 16;
 template <typename T>
 __host__ __device__ inline int vec_chunk_groups(long long n_voxels, int voxels_per_group) {
-    constexpr int kVecMinChunks = sizeof(T) == 4 ? 400 : 1300;
+    constexpr int kVecSlots = 456, kVecMinChunks = 1300;
     const long long per_block = (long long)kThreads * voxels_per_group;
     const long long groups = (n_voxels + per_block - 1) / per_block;
+    if (sizeof(T) == 4) {
+        const long long per = (groups + kVecSlots - 1) / kVecSlots;
+        return per < 1 ? 1 : per < kVecChunkGroups ? (int)per : kVecChunkGroups;
+    }
     int per = kVecChunkGroups;
     while (per > 1 && groups < (long long)kVecMinChunks * per) per /= 2;
     return per;
