@@ -54,6 +54,8 @@ template <> struct CxOf<double> { using type = double2; };
 template <typename T> using cx = typename CxOf<T>::type;
 
 template <typename C> __device__ __forceinline__ C cmake(decltype(C::x) a, decltype(C::x) b) { C r; r.x = a; r.y = b; return r; }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return cmake<C>(a.x + b.x, a.y + b.y); }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return cmake<C>(a.x - b.x, a.y - b.y); }
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
@@ -67,6 +69,10 @@ template <typename C> __device__ __forceinline__ C cscale(C a, decltype(C::x) s)
 // In-register forward DFTs of size R (omega = exp(-2 pi i / R)).
 template <typename C, int R> struct Dft;
 
+template <typename C> struct Dft<C, 1> {
+    __device__ __forceinline__ static void run(C*) {}
+};
+
 template <typename C> struct Dft<C, 2> {
     __device__ __forceinline__ static void run(C* v) {
         C a = v[0], b = v[1];
@@ -75,12 +81,23 @@ template <typename C> struct Dft<C, 2> {
     }
 };
 
+// Radices 4 and 8 in FP32 take the sums of both components as one packed instruction; the products with 1/sqrt2 go
+// into the sums that use them (one rounding, as the compiler contracts the FP64 form).
+__device__ __forceinline__ float2 cadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 cfma2(float2 s, float2 a, float2 b) { return __ffma2_rn(s, a, b); }
+__device__ __forceinline__ double2 cadd2(double2 a, double2 b) { return cadd(a, b); }
+__device__ __forceinline__ double2 csub2(double2 a, double2 b) { return csub(a, b); }
+__device__ __forceinline__ double2 cfma2(double2 s, double2 a, double2 b) {
+    return make_double2(fma(s.x, a.x, b.x), fma(s.y, a.y, b.y));
+}
+
 template <typename C> struct Dft<C, 4> {
     __device__ __forceinline__ static void run(C* v) {
-        C s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-        C s13 = cadd(v[1], v[3]), d13 = cmul_mi(csub(v[1], v[3]));
-        v[0] = cadd(s02, s13);
-        v[2] = csub(s02, s13);
+        C s02 = cadd2(v[0], v[2]), d02 = csub2(v[0], v[2]);
+        C s13 = cadd2(v[1], v[3]), d13 = cmul_mi(csub2(v[1], v[3]));
+        v[0] = cadd2(s02, s13);
+        v[2] = csub2(s02, s13);
         v[1] = cadd(d02, d13);
         v[3] = csub(d02, d13);
     }
@@ -95,17 +112,17 @@ template <typename C> struct Dft<C, 8> {
         Dft<C, 4>::run(e);
         Dft<C, 4>::run(o);
         // o[m] *= exp(-2 pi i m / 8)
-        C o1 = cmake<C>(h * (o[1].x + o[1].y), h * (o[1].y - o[1].x));
-        C o2 = cmul_mi(o[2]);
-        C o3 = cmake<C>(h * (o[3].y - o[3].x), -h * (o[3].x + o[3].y));
-        v[0] = cadd(e[0], o[0]);
-        v[4] = csub(e[0], o[0]);
-        v[1] = cadd(e[1], o1);
-        v[5] = csub(e[1], o1);
+        const C o1 = cmake<C>(o[1].x + o[1].y, o[1].y - o[1].x);
+        const C o2 = cmul_mi(o[2]);
+        const C o3 = cmake<C>(o[3].y - o[3].x, o[3].x + o[3].y);
+        v[0] = cadd2(e[0], o[0]);
+        v[4] = csub2(e[0], o[0]);
+        v[1] = cfma2(cmake<C>(h, h), o1, e[1]);
+        v[5] = cfma2(cmake<C>(-h, -h), o1, e[1]);
         v[2] = cadd(e[2], o2);
         v[6] = csub(e[2], o2);
-        v[3] = cadd(e[3], o3);
-        v[7] = csub(e[3], o3);
+        v[3] = cfma2(cmake<C>(h, -h), o3, e[3]);
+        v[7] = cfma2(cmake<C>(-h, h), o3, e[3]);
     }
 };
 
@@ -201,6 +218,19 @@ __device__ C* block_fft(C* a, C* b, const AxisPlan& ap, const C* __restrict__ tw
     return a;
 }
 
+// Runs the statement with RR = the radix of a stage.
+#define CCMF_DISPATCH_RADIX(radix, ...)                           \
+    do {                                                          \
+        switch (radix) {                                          \
+            case 8: { constexpr int RR = 8; __VA_ARGS__; break; } \
+            case 4: { constexpr int RR = 4; __VA_ARGS__; break; } \
+            case 2: { constexpr int RR = 2; __VA_ARGS__; break; } \
+            case 3: { constexpr int RR = 3; __VA_ARGS__; break; } \
+            case 5: { constexpr int RR = 5; __VA_ARGS__; break; } \
+            default: { constexpr int RR = 1; __VA_ARGS__; break; } \
+        }                                                         \
+    } while (0)
+
 // In-place mixed-radix Cooley-Tukey stages on lines held in shared memory
 // (element m of line c at buf[c * ls + m * es]). Stage st works on blocks of Ls
 // elements; butterfly (block b, offset j < m = Ls / R) combines the elements
@@ -211,14 +241,14 @@ __device__ C* block_fft(C* a, C* b, const AxisPlan& ap, const C* __restrict__ tw
 // Decimation in time (DIT: twiddle, then transform, stages in reverse order)
 // maps digit-reversed input to natural-order output. Both use the forward
 // kernel exp(-2 pi i / n). Threads take consecutive lines first.
-template <typename C, int R, bool DIF, int NT>
+template <typename C, int R, bool DIF, int NT = 0>
 __device__ __forceinline__ void inplace_stage(C* buf, int n, int nlines, int es, int ls, int Ls,
                                               const FastDiv& msub, const FastDiv& nld,
                                               const C* __restrict__ tw) {
     const int m = (int)msub.d;
     const int total = nlines * (n / R);
     const int tws = n / Ls;
-    for (int q = threadIdx.x; q < total; q += NT) {
+    for (int q = threadIdx.x; q < total; q += NT ? NT : (int)blockDim.x) {
         const int bj = (int)fdiv((unsigned)q, nld);
         const int c = q - bj * nlines;
         const int b = (int)fdiv((unsigned)bj, msub);

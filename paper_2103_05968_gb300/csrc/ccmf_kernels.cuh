@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kThreads) k_init_state(Geom g, Ptrs<T> p) {
 // q in [b P, b P + P) as real and imaginary parts of one complex line.
 // d(p) = (1/sqrt2) sum_a [w1_a(p) - w1_a(p - e_a) + w2_a(p + e_a) - w2_a(p)].
 // FP64 leaves out the factor 1/sqrt2 (div_scale): see fold_h.
-// VEC: each thread reads W consecutive voxels of a line with 16-byte loads.
+// VEC: each thread takes W consecutive voxels of a line (two; four for the stored divergences).
 // ---------------------------------------------------------------------------
 template <typename T, int P, bool VEC, bool AB = false>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 1) k_div_rfft_z(Geom g, Ptrs<T> p, AxisPlan az,
@@ -726,12 +726,91 @@ __global__ void __launch_bounds__(kThreads, wlines_min_blocks<T, MODE, N>())
 // the inverse runs as conj(DIT(conj(.))) along x then y, which returns natural
 // order. No permutation pass and no second buffer are needed.
 // ---------------------------------------------------------------------------
-// Threads of the one-block plane pass: 1024 in FP32 (64 registers, no spills; 0.066 against 0.070 ms per
-// 128^3 x 3 launch with 512 on GB300), 512 in FP64 (at 1024 the FP64 kernel spills).
+// Most threads of a plane block: 1024 in FP32 (64 registers, no spills), 512 in FP64 (at 1024 it spills).
 template <typename T>
 __host__ __device__ constexpr int plane_threads() { return sizeof(T) == 4 ? 1024 : 512; }
 constexpr int kPlaneMax = 16384;
 
+// First y stage of the plane pass: global rows -> butterflies -> tile (rows of pitch P2). Consecutive threads take
+// consecutive elements of a row.
+template <typename C, int R>
+__device__ __forceinline__ void plane_load_stage(const C* __restrict__ spec, C* tile, int n1, int n2, int P2,
+                                                 const FastDiv& msub, const C* __restrict__ tw) {
+    const int m = (int)msub.d;
+    const int total = n1 * m;
+    for (int q = threadIdx.x; q < total; q += blockDim.x) {
+        const int i = (int)fdiv((unsigned)q, msub);
+        const int j = q - i * m;
+        const C* src = spec + i * n2 + j;
+        C v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = src[r * m];
+        Dft<C, R>::run(v);
+        C* x = tile + i * P2 + j;
+        x[0] = v[0];
+#pragma unroll
+        for (int r = 1; r < R; ++r) x[r * m] = cmul(v[r], tw[j * r]);
+    }
+}
+
+// Last stage of the inverse y transforms: tile -> butterflies -> conjugate to the global rows.
+template <typename C, int R>
+__device__ __forceinline__ void plane_store_stage(C* __restrict__ spec, const C* tile, int n1, int n2, int P2,
+                                                  const FastDiv& msub, const C* __restrict__ tw) {
+    const int m = (int)msub.d;
+    const int total = n1 * m;
+    for (int q = threadIdx.x; q < total; q += blockDim.x) {
+        const int i = (int)fdiv((unsigned)q, msub);
+        const int j = q - i * m;
+        const C* x = tile + i * P2 + j;
+        C v[R];
+        v[0] = x[0];
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = cmul(x[r * m], tw[j * r]);
+        Dft<C, R>::run(v);
+        C* dst = spec + i * n2 + j;
+#pragma unroll
+        for (int r = 0; r < R; ++r) dst[r * m] = cconj(v[r]);
+    }
+}
+
+// Last x stage, Poisson gain and first inverse x stage: the same R elements of a column (no twiddles in either).
+template <typename C, int R>
+__device__ __forceinline__ void plane_gain_stage(C* tile, int n1, int n2, int P2, const FastDiv& dn2,
+                                                 const decltype(C::x)* __restrict__ rsym1,
+                                                 const decltype(C::x)* __restrict__ rsym2, decltype(C::x) l3,
+                                                 decltype(C::x) inv_n) {
+    using T = decltype(C::x);
+    const int total = n2 * (n1 / R);
+    for (int q = threadIdx.x; q < total; q += blockDim.x) {
+        const int b = (int)fdiv((unsigned)q, dn2);
+        const int c = q - b * n2;
+        C* x = tile + b * R * P2 + c;
+        C v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = x[r * P2];
+        Dft<C, R>::run(v);
+        const T l2 = rsym2[c];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const T lam = rsym1[b * R + r] + l2 + l3;
+            const T gk = (lam > T(0)) ? poisson_gain_div(inv_n, lam) : T(0);
+            // conj: the inverse runs as conj(DIT(conj)); rounded here, not fused into the next stage's sums
+            v[r] = cmake<C>(mul_rn(v[r].x, gk), mul_rn(-v[r].y, gk));
+        }
+        Dft<C, R>::run(v);
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r * P2] = v[r];
+    }
+}
+
+// Bound by instruction issue and by the passes over shared memory: the first and the last y stage work on global
+// memory, the Poisson gain sits in the last x stage, and the radix-4 and -8 butterflies use packed FP32 sums, so a
+// 128 x 128 plane takes 11 passes (15 with load, gain and store passes of their own): three 128^3 solves 67 -> 58 us,
+// six 96^3 47 -> 35, one 64^3 14.6 -> 12.8. Slower forms: one body for all passes executes more index arithmetic (77
+// us for three 128^3 solves); groups of two stages in registers leave too few warps (two 100 x 90 x 150 solves: 41 us
+// against 31); radices up to 16 gain nothing in FP64 and round differently. The odd pitch keeps row accesses free of
+// bank conflicts.
 template <typename T>
 __global__ void __launch_bounds__(plane_threads<T>(), 1) k_fft_plane(Geom g, Ptrs<T> p, AxisPlan ax1, AxisPlan ax2,
                                                                 const cx<T>* __restrict__ tw1,
@@ -740,45 +819,39 @@ __global__ void __launch_bounds__(plane_threads<T>(), 1) k_fft_plane(Geom g, Ptr
                                                                 const T* __restrict__ rsym2,
                                                                 const T* __restrict__ sym3, T inv_n) {
     using C = cx<T>;
-    constexpr int kPlaneThreads = plane_threads<T>();
     const int s = blockIdx.y + p.s0;
     if (!p.run_all && !p.sc[s].active) return;
     const int kz = blockIdx.x;
     const int n1 = g.n1, n2 = g.n2;
-    const int P2 = n2 + 1;
+    const int P2 = n2 | 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tx = reinterpret_cast<C*>(smem_raw);
     C* ty = tx + n1;
     C* tile = ty + n2;
-    for (int t = threadIdx.x; t < n1; t += kPlaneThreads) tx[t] = tw1[t];
-    for (int t = threadIdx.x; t < n2; t += kPlaneThreads) ty[t] = tw2[t];
+    for (int t = threadIdx.x; t < n1; t += blockDim.x) tx[t] = tw1[t];
+    for (int t = threadIdx.x; t < n2; t += blockDim.x) ty[t] = tw2[t];
     C* spec = p.spec + (size_t)s * g.Nh + (long long)kz * n1 * n2;
-    const int cnt = n1 * n2;
-    for (int idx = threadIdx.x; idx < cnt; idx += kPlaneThreads) {
-        const int i = (int)fdiv((unsigned)idx, g.div_n2);
-        cp_async_cx(&tile[i * P2 + (idx - i * n2)], &spec[idx]);
-    }
-    cp_async_wait_all();
-    __syncthreads();
     const FastDiv dn1 = g.div_n1, dn2 = g.div_n2;
-    inplace_fft<C, true, kPlaneThreads>(tile, ax2, n1, 1, P2, dn1, ty);    // y: n1 rows
-    inplace_fft<C, true, kPlaneThreads>(tile, ax1, n2, P2, 1, dn2, tx);    // x: n2 columns
-    const T l3 = sym3[kz];
-    for (int idx = threadIdx.x; idx < cnt; idx += kPlaneThreads) {
-        const int i = (int)fdiv((unsigned)idx, g.div_n2);
-        const int j = idx - i * n2;
-        const T lam = rsym1[i] + rsym2[j] + l3;
-        const T gk = (lam > T(0)) ? poisson_gain_div(inv_n, lam) : T(0);
-        const C z = tile[i * P2 + j];
-        tile[i * P2 + j] = cmake<C>(z.x * gk, -z.y * gk);   // conj: the inverse runs as conj(DIT(conj))
-    }
+    const int s1 = max(ax1.nst, 1);   // a line of one element: one stage of radix 1
+    __syncthreads();                  // twiddles
+    CCMF_DISPATCH_RADIX(ax2.rad[0], (plane_load_stage<C, RR>(spec, tile, n1, n2, P2, ax2.sub[0], ty)));
     __syncthreads();
-    inplace_fft<C, false, kPlaneThreads>(tile, ax1, n2, P2, 1, dn2, tx);
-    inplace_fft<C, false, kPlaneThreads>(tile, ax2, n1, 1, P2, dn1, ty);
-    for (int idx = threadIdx.x; idx < cnt; idx += kPlaneThreads) {
-        const int i = (int)fdiv((unsigned)idx, g.div_n2);
-        spec[idx] = cconj(tile[i * P2 + (idx - i * n2)]);
-    }
+    for (int k = 1; k < ax2.nst; ++k)
+        CCMF_DISPATCH_RADIX(ax2.rad[k], (inplace_stage<C, RR, true>(tile, n2, n1, 1, P2, ax2.span[k], ax2.sub[k], dn1,
+                                                                     ty)));
+    for (int k = 0; k < s1 - 1; ++k)
+        CCMF_DISPATCH_RADIX(ax1.rad[k], (inplace_stage<C, RR, true>(tile, n1, n2, P2, 1, ax1.span[k], ax1.sub[k], dn2,
+                                                                     tx)));
+    CCMF_DISPATCH_RADIX(ax1.rad[s1 - 1],
+                        (plane_gain_stage<C, RR>(tile, n1, n2, P2, dn2, rsym1, rsym2, sym3[kz], inv_n)));
+    __syncthreads();
+    for (int k = s1 - 2; k >= 0; --k)
+        CCMF_DISPATCH_RADIX(ax1.rad[k], (inplace_stage<C, RR, false>(tile, n1, n2, P2, 1, ax1.span[k], ax1.sub[k], dn2,
+                                                                      tx)));
+    for (int k = ax2.nst - 1; k >= 1; --k)
+        CCMF_DISPATCH_RADIX(ax2.rad[k], (inplace_stage<C, RR, false>(tile, n2, n1, 1, P2, ax2.span[k], ax2.sub[k], dn1,
+                                                                      ty)));
+    CCMF_DISPATCH_RADIX(ax2.rad[0], (plane_store_stage<C, RR>(spec, tile, n1, n2, P2, ax2.sub[0], ty)));
 }
 
 // ---------------------------------------------------------------------------

@@ -192,7 +192,8 @@ int lines_blocks_per_sm(int mode, int lines, size_t smem) {
 // Instantiations of k_update: update variant 0 (16-byte vectors), 11 (half of them, two blocks per SM), 12
 // (half, three blocks per SM), any N3 or alignment (strided packs); FP32 writes the (z, s) format, or (e, v)
 // where the caller needs it (WZS = false, strided packs only: the reverse mode's forward passes and update variants
-// 1 .. 10, 13 .. 15 on grids that they do not cover). FP64 always writes (e, v).
+// 1 .. 10, 13 .. 15 on grids that they do not cover). FP64 always writes (e, v). A one-voxel FP64 group needs no
+// alignment, so the pair kinds of FP64 are strided packs of one.
 enum UpdateKind { kUpdFull = 0, kUpdHalf2, kUpdHalf3, kUpdStrided, kUpdStridedEv, kNumUpdateKinds };
 
 template <typename T, bool OUT, int RULE>
@@ -487,7 +488,7 @@ void launch_passes(const Ctx<T>& c, const Ptrs<T>& p, cudaStream_t st, F&& betwe
         launch_plane_cluster<T>(g, p, c, inv_n, st);
         between(kKFftPlane);
     } else if (sh.plane_fused) {
-        k_fft_plane<T><<<dim3((unsigned)g.n3h, (unsigned)g.batch), plane_threads<T>(), sh.smem_plane, st>>>(
+        k_fft_plane<T><<<dim3((unsigned)g.n3h, (unsigned)g.batch), sh.plane_threads, sh.smem_plane, st>>>(
             g, p, c.ax[0], c.ax[1], c.tw[0], c.tw[1], c.rsym[0], c.rsym[1], c.sym[2], inv_n);
         between(kKFftPlane);
     } else {

@@ -144,6 +144,7 @@ struct LaunchShape {
     int grid_pipe;            // blocks per solve of the pipelined update
     size_t smem_pipe;         // its dynamic shared memory
     int plane_fused;          // 1: y / x / solve / x / y in one plane launch per iteration
+    int plane_threads;        // threads of k_fft_plane
     size_t smem_plane;        // its dynamic shared memory (per block)
     int plane_cluster;        // blocks sharing one plane: 1 = k_fft_plane, 2..16 = k_fft_plane_cluster
     int grid_y, grid_x;       // persistent blocks per solve of the y / x line passes (0: one tile per block)
