@@ -423,9 +423,10 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     if (explicit_variant && sh.upd_variant != variant) return CCMF_ERR_UNSUPPORTED_SIZE;
     r.update_variant = sh.upd_variant;
     {
-        const int kind = sh.upd_variant == 11 || sh.upd_variant == 12
-                             ? (n3 % 2 != 0 ? kUpdStrided : sh.upd_variant == 11 ? kUpdHalf2 : kUpdHalf3)
-                             : (n3 % W != 0 ? kUpdStrided : kUpdFull);
+        const int kind = n3 % 2 != 0 ? kUpdStrided
+                         : sh.upd_variant == 11 ? kUpdHalf2
+                         : sh.upd_variant == 12 || n3 % W != 0 ? kUpdHalf3
+                                                               : kUpdFull;
         const int okind = n3 % W != 0 ? kUpdStrided : kUpdFull;
         sh.upd_resident = (f64 ? update_blocks_per_sm<double>(kind, false) : update_blocks_per_sm<float>(kind, false)) * sms;
         sh.out_resident = (f64 ? update_blocks_per_sm<double>(okind, true) : update_blocks_per_sm<float>(okind, true)) * sms;

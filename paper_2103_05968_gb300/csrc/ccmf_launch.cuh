@@ -237,9 +237,10 @@ int update_blocks_per_sm(int kind, bool out) {
 template <typename T>
 int update_kind(const Ctx<T>& c) {
     if (sizeof(T) == 4 && !c.use_zs) return kUpdStridedEv;
-    if (c.sh.upd_variant == 11 || c.sh.upd_variant == 12)
-        return !c.pair_update ? kUpdStrided : c.sh.upd_variant == 11 ? kUpdHalf2 : kUpdHalf3;
-    return c.vec_update ? kUpdFull : kUpdStrided;
+    if (!c.pair_update) return kUpdStrided;
+    if (c.sh.upd_variant == 11) return kUpdHalf2;
+    // variant 12, and every N3 = 2 mod 4 (where the plan resolves to variant 0)
+    return c.sh.upd_variant == 12 || !c.vec_update ? kUpdHalf3 : kUpdFull;
 }
 
 #define CCMF_DISPATCH_ABW(var, ...)                                                      \
