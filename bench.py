@@ -153,20 +153,22 @@ def basis_bytes_per_voxel(esize):
     return 33 * esize
 
 
-def bytes_per_voxel(kernel, esize, n3, stored_div=False):
+def bytes_per_voxel(kernel, esize, n3, stored_div=False, compact=False):
     """Algorithmic DRAM bytes per voxel of one launch of each loop kernel. stored_div: the
     stored-divergence schedule (update variants 8 - 10), whose first pass reads the two
-    divergences a, b and whose update pass also writes them."""
+    divergences a, b and whose update pass also writes them. compact: the (z, s) state (seven
+    values in place of the twelve of e, v)."""
+    state = 7 if compact else 12
     half = (n3 // 2 + 1) / n3 * 2 * esize  # half-spectrum bytes per voxel
     return {
-        "k_div_rfft_z": (2 if stored_div else 12) * esize + half,   # read a, b (or e, v); write spectrum
+        "k_div_rfft_z": (2 if stored_div else state) * esize + half,   # read a, b (or the state); write spectrum
         "k_fft_y_fwd": 2 * half,                    # read + write spectrum
         "k_fft_x_solve": 2 * half,
         "k_fft_y_inv": 2 * half,
         "k_fft_plane": 2 * half,                    # read + write spectrum once (y, x, solve, x, y fused)
         "k_irfft_z": half + esize,                  # read spectrum; write phi
-        # read e, v, gamma, phi; write e, v (and a, b)
-        "k_update": 12 * esize + 2 * esize + 12 * esize + (2 * esize if stored_div else 0),
+        # read the state, gamma, phi; write the state (and a, b)
+        "k_update": state * esize + 2 * esize + state * esize + (2 * esize if stored_div else 0),
     }[kernel]
 
 
@@ -176,10 +178,16 @@ def plan_stored_div(plan):
     return 8 <= v <= 10 or 13 <= v <= 15
 
 
+def plan_compact(plan, esize):
+    """True when the update pass keeps the (z, s) state: FP32 with update variant 0, 11 or 12."""
+    return esize == 4 and int(plan.tuning()["update_variant"]) in (0, 11, 12)
+
+
 def load_traffic(kernel, workload, precision, with_source=False):
     """DRAM bytes per launch of a kernel from the committed ncu summaries (profiles/*.md),
     or None when no capture of this kernel, workload and precision is recorded. The
-    update pass is keyed with its variant (k_update@v<variant>), so a figure measured on
+    update pass is keyed with its variant (k_update@v<variant>, k_update@zs<variant> on the
+    compact state), so a figure measured on
     one variant is never reported for another. with_source: also return the file name."""
     import glob
     for path in sorted(glob.glob(os.path.join(ROOT, "profiles", "*.md"))):
@@ -419,8 +427,8 @@ def fibres512_record(args, dev):
     peak, peak_kind = load_peaks()
     dom = max(kt, key=lambda k: kt[k][0])
     dom_ms = kt[dom][0] / kt[dom][1]
-    sd = plan_stored_div(plan)
-    dom_bytes = bytes_per_voxel(dom, 4, 512, sd) * N
+    sd, zs = plan_stored_div(plan), plan_compact(plan, 4)
+    dom_bytes = bytes_per_voxel(dom, 4, 512, sd, zs) * N
     basis = basis_bytes_per_voxel(4) * N
     ms_step, ms_iter = t_k / K, (t_2k - t_k) / K
     tuning = plan.tuning()
@@ -434,7 +442,7 @@ def fibres512_record(args, dev):
                                 "achieved_gbs": dom_bytes / (dom_ms * 1e-3) / 1e9,
                                 "frac": dom_bytes / (dom_ms * 1e-3) / 1e9 / peak},
             "kernels_ms_per_launch": {k: v[0] / v[1] for k, v in kt.items()},
-            "own_schedule_bytes_per_voxel": sum(bytes_per_voxel(k, 4, 512, sd) for k in kt),
+            "own_schedule_bytes_per_voxel": sum(bytes_per_voxel(k, 4, 512, sd, zs) for k in kt),
             "tuning": tuning,
             "peak": peak, "peak_kind": peak_kind, "autotune": tune, "setup_seconds": setup_s,
             "l2": "inputs larger than L2: state 6.4 GB per step"}
@@ -742,16 +750,16 @@ def run_gpu(args, world, rank, local):
     # roofline of the dominant kernel
     dom = max(kt, key=lambda k: kt[k][0])
     dom_ms, dom_n = kt[dom]
-    sd = plan_stored_div(plan)
-    per_launch_bytes = bytes_per_voxel(dom, esize, n3, sd) * N * B
+    sd, zs = plan_stored_div(plan), plan_compact(plan, esize)
+    per_launch_bytes = bytes_per_voxel(dom, esize, n3, sd, zs) * N * B
     achieved = per_launch_bytes / (dom_ms / dom_n * 1e-3) / 1e9
     peak, peak_kind = load_peaks()
     kern = {k: {"ms_per_launch": ms / n, "launches": n, "share": ms / sum(x[0] for x in kt.values()),
-                "gbs": bytes_per_voxel(k, esize, n3, sd) * N * B / (ms / n * 1e-3) / 1e9}
+                "gbs": bytes_per_voxel(k, esize, n3, sd, zs) * N * B / (ms / n * 1e-3) / 1e9}
             for k, (ms, n) in kt.items()}
-    own_bpv = sum(bytes_per_voxel(k, esize, n3, sd) for k in kt)
+    own_bpv = sum(bytes_per_voxel(k, esize, n3, sd, zs) for k in kt)
     tuned = plan.tuning()
-    traffic_key = f"{dom}@v{tuned['update_variant']}" if dom == "k_update" else dom
+    traffic_key = f"{dom}@{'zs' if zs else 'v'}{tuned['update_variant']}" if dom == "k_update" else dom
     traffic, traffic_src = (None, None) if args.grid else load_traffic(traffic_key, name, args.precision,
                                                                        with_source=True)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,

@@ -201,7 +201,9 @@ int ccmf_plan_launch_info(const ccmf_plan* plan, int* out, int capacity, int* co
  * In ccmf_plan_set_tuning a negative entry selects the built-in rule.
  */
 typedef struct {
-    int update_variant;     /* update pass: 0 register vectors in ticket-ordered chunks, 1 TMA rows,
+    int update_variant;     /* update pass: 0 register vectors in ticket-ordered chunks (as 11 and 12
+                               it keeps the FP32 state as z and the projection factor s, 7 values
+                               per voxel in place of the 12 of e, v), 1 TMA rows,
                                2..7 pipelined TMA; 8, 9 the stored-divergence schedule: the update
                                pass also writes a = div^- A* e and b = div^- A* v of the new state
                                (Eq. 28, Eq. 30: the divergence of e - v / rho is a - b / rho), so the
