@@ -81,23 +81,12 @@ template <typename C> struct Dft<C, 2> {
     }
 };
 
-// Radices 4 and 8 in FP32 take the sums of both components as one packed instruction; the products with 1/sqrt2 go
-// into the sums that use them (one rounding, as the compiler contracts the FP64 form).
-__device__ __forceinline__ float2 cadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 csub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ float2 cfma2(float2 s, float2 a, float2 b) { return __ffma2_rn(s, a, b); }
-__device__ __forceinline__ double2 cadd2(double2 a, double2 b) { return cadd(a, b); }
-__device__ __forceinline__ double2 csub2(double2 a, double2 b) { return csub(a, b); }
-__device__ __forceinline__ double2 cfma2(double2 s, double2 a, double2 b) {
-    return make_double2(fma(s.x, a.x, b.x), fma(s.y, a.y, b.y));
-}
-
 template <typename C> struct Dft<C, 4> {
     __device__ __forceinline__ static void run(C* v) {
-        C s02 = cadd2(v[0], v[2]), d02 = csub2(v[0], v[2]);
-        C s13 = cadd2(v[1], v[3]), d13 = cmul_mi(csub2(v[1], v[3]));
-        v[0] = cadd2(s02, s13);
-        v[2] = csub2(s02, s13);
+        C s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
+        C s13 = cadd(v[1], v[3]), d13 = cmul_mi(csub(v[1], v[3]));
+        v[0] = cadd(s02, s13);
+        v[2] = csub(s02, s13);
         v[1] = cadd(d02, d13);
         v[3] = csub(d02, d13);
     }
@@ -112,17 +101,17 @@ template <typename C> struct Dft<C, 8> {
         Dft<C, 4>::run(e);
         Dft<C, 4>::run(o);
         // o[m] *= exp(-2 pi i m / 8)
-        const C o1 = cmake<C>(o[1].x + o[1].y, o[1].y - o[1].x);
-        const C o2 = cmul_mi(o[2]);
-        const C o3 = cmake<C>(o[3].y - o[3].x, o[3].x + o[3].y);
-        v[0] = cadd2(e[0], o[0]);
-        v[4] = csub2(e[0], o[0]);
-        v[1] = cfma2(cmake<C>(h, h), o1, e[1]);
-        v[5] = cfma2(cmake<C>(-h, -h), o1, e[1]);
+        C o1 = cmake<C>(h * (o[1].x + o[1].y), h * (o[1].y - o[1].x));
+        C o2 = cmul_mi(o[2]);
+        C o3 = cmake<C>(h * (o[3].y - o[3].x), -h * (o[3].x + o[3].y));
+        v[0] = cadd(e[0], o[0]);
+        v[4] = csub(e[0], o[0]);
+        v[1] = cadd(e[1], o1);
+        v[5] = csub(e[1], o1);
         v[2] = cadd(e[2], o2);
         v[6] = csub(e[2], o2);
-        v[3] = cfma2(cmake<C>(h, -h), o3, e[3]);
-        v[7] = cfma2(cmake<C>(-h, h), o3, e[3]);
+        v[3] = cadd(e[3], o3);
+        v[7] = csub(e[3], o3);
     }
 };
 
@@ -163,6 +152,50 @@ template <typename C> struct Dft<C, 5> {
     }
 };
 
+// The same DFTs for the block stages, whose inputs come from memory: radices 4 and 8 in FP32 take the sums of both
+// components as one packed instruction, and the products with 1/sqrt2 go into the sums that use them, which is how
+// the compiler contracts Dft, so the results are the same bits. (The warp FFTs keep Dft: there the compiler also
+// contracts the caller's products, the Poisson gain, into the first sums.)
+template <typename C, int R> struct DftBlock : Dft<C, R> {};
+__device__ __forceinline__ float2 cadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 cfma2(float2 s, float2 a, float2 b) { return __ffma2_rn(s, a, b); }
+
+template <> struct DftBlock<float2, 4> {
+    using C = float2;
+    __device__ __forceinline__ static void run(C* v) {
+        C s02 = cadd2(v[0], v[2]), d02 = csub2(v[0], v[2]);
+        C s13 = cadd2(v[1], v[3]), d13 = cmul_mi(csub2(v[1], v[3]));
+        v[0] = cadd2(s02, s13);
+        v[2] = csub2(s02, s13);
+        v[1] = cadd(d02, d13);
+        v[3] = csub(d02, d13);
+    }
+};
+
+template <> struct DftBlock<float2, 8> {
+    using C = float2;
+    __device__ __forceinline__ static void run(C* v) {
+        const float h = 0.70710678118654752440084436210485f;
+        C e[4] = {v[0], v[2], v[4], v[6]};
+        C o[4] = {v[1], v[3], v[5], v[7]};
+        DftBlock<C, 4>::run(e);
+        DftBlock<C, 4>::run(o);
+        // o[m] *= exp(-2 pi i m / 8)
+        const C o1 = cmake<C>(o[1].x + o[1].y, o[1].y - o[1].x);
+        const C o2 = cmul_mi(o[2]);
+        const C o3 = cmake<C>(o[3].y - o[3].x, o[3].x + o[3].y);
+        v[0] = cadd2(e[0], o[0]);
+        v[4] = csub2(e[0], o[0]);
+        v[1] = cfma2(cmake<C>(h, h), o1, e[1]);
+        v[5] = cfma2(cmake<C>(-h, -h), o1, e[1]);
+        v[2] = cadd(e[2], o2);
+        v[6] = csub(e[2], o2);
+        v[3] = cfma2(cmake<C>(h, -h), o3, e[3]);
+        v[7] = cfma2(cmake<C>(-h, h), o3, e[3]);
+    }
+};
+
 // One Stockham stage of radix R over LINES lines (LINES a power of two):
 // butterfly j of line c reads elements j + r n/R, applies the twiddles
 // W_{Ns R}^{(j mod Ns) r}, transforms, and writes to
@@ -189,7 +222,7 @@ __device__ __forceinline__ void stockham_stage(const C* __restrict__ src, C* __r
 #pragma unroll
             for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[t * r]);
         }
-        Dft<C, R>::run(v);
+        DftBlock<C, R>::run(v);
         const int od = (j - jm) * R + jm;
 #pragma unroll
         for (int r = 0; r < R; ++r) dst[(od + r * Ns) * stride + c] = v[r];
@@ -258,7 +291,7 @@ __device__ __forceinline__ void inplace_stage(C* buf, int n, int nlines, int es,
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = x[r * m * es];
         if (DIF) {
-            Dft<C, R>::run(v);
+            DftBlock<C, R>::run(v);
             if (j > 0) {
 #pragma unroll
                 for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[j * r * tws]);
@@ -268,7 +301,7 @@ __device__ __forceinline__ void inplace_stage(C* buf, int n, int nlines, int es,
 #pragma unroll
                 for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[j * r * tws]);
             }
-            Dft<C, R>::run(v);
+            DftBlock<C, R>::run(v);
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) x[r * m * es] = v[r];

@@ -745,7 +745,7 @@ __device__ __forceinline__ void plane_load_stage(const C* __restrict__ spec, C* 
         C v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = src[r * m];
-        Dft<C, R>::run(v);
+        DftBlock<C, R>::run(v);
         C* x = tile + i * P2 + j;
         x[0] = v[0];
 #pragma unroll
@@ -767,7 +767,7 @@ __device__ __forceinline__ void plane_store_stage(C* __restrict__ spec, const C*
         v[0] = x[0];
 #pragma unroll
         for (int r = 1; r < R; ++r) v[r] = cmul(x[r * m], tw[j * r]);
-        Dft<C, R>::run(v);
+        DftBlock<C, R>::run(v);
         C* dst = spec + i * n2 + j;
 #pragma unroll
         for (int r = 0; r < R; ++r) dst[r * m] = cconj(v[r]);
@@ -789,7 +789,7 @@ __device__ __forceinline__ void plane_gain_stage(C* tile, int n1, int n2, int P2
         C v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = x[r * P2];
-        Dft<C, R>::run(v);
+        DftBlock<C, R>::run(v);
         const T l2 = rsym2[c];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -798,7 +798,7 @@ __device__ __forceinline__ void plane_gain_stage(C* tile, int n1, int n2, int P2
             // conj: the inverse runs as conj(DIT(conj)); rounded here, not fused into the next stage's sums
             v[r] = cmake<C>(mul_rn(v[r].x, gk), mul_rn(-v[r].y, gk));
         }
-        Dft<C, R>::run(v);
+        DftBlock<C, R>::run(v);
 #pragma unroll
         for (int r = 0; r < R; ++r) x[r * P2] = v[r];
     }
