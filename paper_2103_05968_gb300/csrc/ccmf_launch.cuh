@@ -194,6 +194,8 @@ int lines_blocks_per_sm(int mode, int lines, size_t smem) {
 // where the caller needs it (WZS = false, strided packs only: the reverse mode's forward passes and update variants
 // 1 .. 10, 13 .. 15 on grids that they do not cover). FP64 always writes (e, v). A one-voxel FP64 group needs no
 // alignment, so the pair kinds of FP64 are strided packs of one.
+// Strided pairs in FP32: three blocks per SM in spite of 176 bytes of spills (two 90 x 100 x 75 solves 85 us an
+// iteration, 88 with two blocks and no spills); FP64 keeps two.
 enum UpdateKind { kUpdFull = 0, kUpdHalf2, kUpdHalf3, kUpdStrided, kUpdStridedEv, kNumUpdateKinds };
 
 template <typename T, bool OUT, int RULE>
@@ -209,7 +211,7 @@ const void* update_kernel(int kind) {
             case kUpdFull: return (const void*)k_update<T, WF, false, RULE, F, 1>;
             case kUpdHalf2: return (const void*)k_update<T, WH, false, RULE, F, 2>;
             case kUpdHalf3: return (const void*)k_update<T, WH, false, RULE, F, 3>;
-            case kUpdStrided: return (const void*)k_update<T, 0, false, RULE, F, 2>;
+            case kUpdStrided: return (const void*)k_update<T, 0, false, RULE, F, F ? 3 : 2>;
             default: return (const void*)k_update<T, 0, false, F ? -1 : RULE, false, 2>;
         }
     }
