@@ -692,8 +692,7 @@ Ctx<T> make_ctx(const ccmf_plan* pl, unsigned char* ws, const T* gamma, long lon
     // table is aligned by the batch API's allocations of whole fields)
     c.use_ab = is_ab_variant(pl->sh.upd_variant) && c.vec_update;
     // the register update variants of FP32 write the (z, s) state; the others read and write (e, v)
-    set_state_format(&c, sizeof(T) == 4 && (pl->sh.upd_variant == 0 || pl->sh.upd_variant == 11 ||
-                                            pl->sh.upd_variant == 12));
+    set_state_format(&c, sizeof(T) == 4 && is_register_variant(pl->sh.upd_variant));
     return c;
 }
 
@@ -2101,6 +2100,16 @@ AdjLayout adj_layout(const ccmf_plan* pl, int K, int m) {
     return L;
 }
 
+// The passes of the reverse mode's forward replay and recomputation, whatever update variant the plan is tuned to:
+// checkpoints hold (e, v), and only the register update pass (variants 0, 11, 12) writes z = v + rho xi (Ptrs::zout),
+// which the reverse steps read.
+template <typename T>
+void set_adjoint_passes(Ctx<T>* c) {
+    c->use_ab = false;
+    if (!is_register_variant(c->sh.upd_variant)) c->sh.upd_variant = 0;
+    set_state_format(c, false);
+}
+
 template <typename T>
 int adjoint_impl(ccmf_plan* pl, const T* gamma, long long gstride, const double* xi_host, const ccmf_params* prm,
                  int K, int m, const double* sched_host, unsigned char* ws, unsigned char* aws, T* grad,
@@ -2160,8 +2169,7 @@ int adjoint_impl(ccmf_plan* pl, const T* gamma, long long gstride, const double*
     cfg.rho_sched = dsched;
     cfg.sched_len = K;
     Ctx<T> c = make_ctx<T>(pl, ws, gamma, gstride, cfg);
-        c.use_ab = false;
-    set_state_format(&c, false);   // checkpoints of (e, v)
+    set_adjoint_passes(&c);
     const size_t f6 = (size_t)6 * g.N * B;
     T* ckpt = reinterpret_cast<T*>(aws + L.ckpt);
     T* e_state = reinterpret_cast<T*>(ws + pl->off_e);
@@ -2397,8 +2405,7 @@ int adjoint_mixed_impl(ccmf_plan* pl, const float* gamma, long long gstride, con
 
     // FP64 forward replay with FP64 checkpoints of (e, v)
     Ctx<double> c64 = make_ctx<double>(p64, ws64, gam64, gstride64, cfg);
-        c64.use_ab = false;
-    set_state_format(&c64, false);
+    set_adjoint_passes(&c64);
     const size_t f6 = (size_t)6 * N * B;
     double* ckpt = reinterpret_cast<double*>(aws + L.ckpt);
     double* e_state = reinterpret_cast<double*>(ws64 + p64->off_e);
@@ -2441,8 +2448,7 @@ int adjoint_mixed_impl(ccmf_plan* pl, const float* gamma, long long gstride, con
 
     // FP32 reverse sweep; the FP32 context supplies the M applications and the seed
     Ctx<float> c32 = make_ctx<float>(pl, ws, gamma, gstride, cfg);
-    c32.use_ab = false;
-    set_state_format(&c32, false);
+    set_adjoint_passes(&c32);
     launch_init<float>(c32, st);   // unit normals and gamma statistics of the FP32 workspace
     float* zbuf = reinterpret_cast<float*>(aws + L.z);
     unsigned* bits = reinterpret_cast<unsigned*>(aws + L.bits);

@@ -185,5 +185,7 @@ constexpr int kNumUpdateVariants = 16;
 __host__ __device__ constexpr bool is_abw_variant(int v) { return v >= 13 && v <= 15; }
 // update variants that write the stored divergences: 8 .. 10 (block-cooperative), 13 .. 15 (warp-independent)
 __host__ __device__ constexpr bool is_ab_variant(int v) { return (v >= 8 && v <= 10) || is_abw_variant(v); }
+// Update variants that run on k_update.
+__host__ __device__ constexpr bool is_register_variant(int v) { return v == 0 || v == 11 || v == 12; }
 
 }  // namespace ccmf
