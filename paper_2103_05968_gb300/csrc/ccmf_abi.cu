@@ -654,6 +654,16 @@ void set_state_format(Ctx<T>* c, bool zs) {
     c->p.zs = zs ? 1 : 0;
 }
 
+// The passes that read gamma with vector loads, from the alignment that the gamma fields of all solves share: the
+// 16-byte update pass, the pairs of the update pass and the stored-divergence schedule (update variants 8 .. 10,
+// 13 .. 15).
+template <typename T>
+void set_gamma_alignment(Ctx<T>* c, bool vec, bool pair) {
+    c->vec_update = c->g.n3 % (16 / (int)sizeof(T)) == 0 && vec;
+    c->pair_update = c->vec_div && pair;
+    c->use_ab = is_ab_variant(c->sh.upd_variant) && c->vec_update;
+}
+
 template <typename T>
 Ctx<T> make_ctx(const ccmf_plan* pl, unsigned char* ws, const T* gamma, long long gstride, const LoopConfig& cfg) {
     Ctx<T> c;
@@ -683,14 +693,13 @@ Ctx<T> make_ctx(const ccmf_plan* pl, unsigned char* ws, const T* gamma, long lon
     c.p.cut = nullptr;
     c.p.flow = nullptr;
     c.p.run_all = 0;
-    const int W = 16 / (int)sizeof(T);
     c.vec_div = (pl->n3 % kDivW) == 0;
-    c.vec_update = (pl->n3 % W) == 0 && ((uintptr_t)gamma % 16) == 0;
-    c.pair_update = c.vec_div && ((uintptr_t)gamma % (2 * sizeof(T))) == 0;
     c.p.ab = reinterpret_cast<T*>(ws + pl->off_ab);
-    // the stored-divergence schedule needs the vector loads of gamma (a per-solve pointer
-    // table is aligned by the batch API's allocations of whole fields)
-    c.use_ab = is_ab_variant(pl->sh.upd_variant) && c.vec_update;
+    // solve s reads gamma + s gstride
+    auto aligned = [&](size_t bytes) {
+        return (uintptr_t)gamma % bytes == 0 && (pl->batch == 1 || (size_t)gstride * sizeof(T) % bytes == 0);
+    };
+    set_gamma_alignment(&c, aligned(16), aligned(2 * sizeof(T)));
     // the register update variants of FP32 write the (z, s) state; the others read and write (e, v)
     set_state_format(&c, sizeof(T) == 4 && is_register_variant(pl->sh.upd_variant));
     return c;

@@ -1,5 +1,7 @@
 """Which kernels the entry points launch, on the stand-in CUDA runtime (CPU)."""
 
+import re
+
 import pytest
 
 from fake_cuda import needs_toolchain, run_fake
@@ -46,3 +48,41 @@ out["kernels"] = [k for _, k, _, _ in launches()]
     # 4 replayed, 1 final evaluation, 4 recomputed, and the final evaluation of each of 4 reverse steps
     assert len(updates) == 13
     assert all("8k_updateI" in k for k in updates), sorted(set(updates))
+
+
+# kernels that load gamma in vectors: k_update on 2 or 4 voxels, the TMA and stored-divergence updates
+_VECTOR = r"8k_updateI[fd]Li[24]E|k_update_(pipe|tma|ab|abw)I"
+
+
+def _vector_kernels(names):
+    return sorted({k for k in names if re.search(_VECTOR, k)})
+
+
+@pytest.mark.parametrize("double", [False, True])
+@pytest.mark.parametrize("variant", [None, 0, 3, 9, 13])
+@pytest.mark.parametrize("call", ["solve", "adjoint"])
+def test_odd_gamma_stride_takes_scalar_loads(call, variant, double, tmp_path):
+    """Field s of a batch starts at gamma + s stride: with an odd stride every second field is off the alignment of a
+    pair, though the base address and N3 are even."""
+    body = _PLAN + f"""
+N = 6 * 8 * 128
+K = 2
+prm = ccmf.Params(fixed_iters=K).to_c()
+def names(batch, stride):
+    h, n = plan_for((6, 8, 128), batch, ccmf.CCMF_FP64 if {double} else ccmf.CCMF_FP32_MIXED)
+    an = ccmf.ccmf_adjoint_workspace_bytes(h, K, K)[1]
+    xi = [[0.0, 0.6, 0.8]] * batch
+    launches()
+    if {call!r} == "solve":
+        code = ccmf.ccmf_solve(h, buf(8 * batch * (N + 1)), stride, xi, prm, buf(n), n, None, None, None, None)
+    else:
+        code = ccmf.ccmf_adjoint(h, buf(8 * batch * (N + 1)), stride, xi, prm, K, K, np.full((batch, K), 0.5), buf(n),
+                                 n, buf(an), an, buf(8 * batch * N), None, None, None)
+    assert code == 0, code
+    return [k for _, k, _, _ in launches()]
+out["one"], out["even"], out["odd"] = names(1, N + 1), names(2, N), names(2, N + 1)
+"""
+    got = run_fake(body, tmp_path, env={} if variant is None else {"CCMF_UPDATE_VARIANT": str(variant)})
+    assert _vector_kernels(got["odd"]) == []
+    assert got["one"] and got["even"]
+    assert _vector_kernels(got["even"]) == _vector_kernels(got["one"]) != []
