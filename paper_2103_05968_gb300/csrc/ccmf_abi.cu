@@ -1728,8 +1728,7 @@ int batch_solve_impl(ccmf_batch* bt, const void* const* gammas, const double* xi
         set_state_format(&ctx[b], bt->persistent ? sizeof(T) == 4 : ctx[b].use_zs);   // the format k_batch_persist runs
     }
     for (int b = 0; b < nb; ++b) {
-        ctx[b].vec_update = bt->plans[b]->n3 % (16 / (int)sizeof(T)) == 0 && aligned;
-        ctx[b].pair_update = ctx[b].vec_div && aligned;
+        set_gamma_alignment(&ctx[b], aligned, aligned);
         launch_init<T>(ctx[b], st);
     }
     if (cudaGetLastError() != cudaSuccess) return CCMF_ERR_CUDA;
@@ -1835,8 +1834,7 @@ int batch_time_bucket(ccmf_batch* bt, int b, unsigned char* ws, bool aligned, in
     cfg.resume = 1;
     Ctx<T> c = make_ctx<T>(pl, wsb, nullptr, 0, cfg);
     c.p.gptrs = reinterpret_cast<const T* const*>(ws + bt->gp_off[b]);
-    c.vec_update = pl->n3 % (16 / (int)sizeof(T)) == 0 && aligned;
-    c.pair_update = c.vec_div && aligned;
+    set_gamma_alignment(&c, aligned, aligned);
     if (cudaMemsetAsync(wsb + pl->off_nact, 0, sizeof(int), st) != cudaSuccess) return CCMF_ERR_CUDA;
     launch_init<T>(c, st);   // resume: re-activates the solves without touching their state
     cudaGraph_t graph;

@@ -72,3 +72,34 @@ def test_padded_batch_with_an_odd_stride(shape, variant, precision):
     for want, got in zip(*out):
         assert torch.isfinite(want).all()
         assert torch.equal(want, got)
+
+
+# The fields are the same bits again; the reported numbers are sums in another grouping, a few eps of each sum: 1e-5 in
+# FP32, 1e-12 in FP64. (The residual is a mean of squares of differences; it is compared at the same bar of |<v>|.)
+@pytest.mark.parametrize("precision,bar", [(ccmf.CCMF_FP64, 1e-12), (ccmf.CCMF_FP32_MIXED, 1e-5)])
+@pytest.mark.parametrize("variant", [None, 3, 9, 13])
+def test_batch_with_an_unaligned_gamma(variant, precision, bar, monkeypatch):
+    if variant is not None:
+        monkeypatch.setenv("CCMF_UPDATE_VARIANT", str(variant))
+    dt = torch.float64 if precision == ccmf.CCMF_FP64 else torch.float32
+    shapes = [(6, 8, 128), (6, 8, 128), (5, 9, 15), (6, 5, 10)]
+    fields = [torch.from_numpy(M.uniform_random(sh, 0.5, 1.5, s)).to(DEV, dt) for s, sh in enumerate(shapes)]
+    normals = np.array([NORMALS[0], NORMALS[1], NORMALS[0], NORMALS[1]])
+    prm = ccmf.Params(fixed_iters=5, rho_rule=ccmf.CCMF_RHO_CONST, rho0=0.4)
+    out = []
+    for offset, persistent in ((0, False), (1, False), (0, True), (1, True)):
+        gammas = []
+        for f in fields:
+            buf = torch.zeros(f.numel() + offset, dtype=dt, device=DEV)
+            buf[offset:] = f.flatten()
+            gammas.append(buf[offset:])
+        batch = ccmf.Batch(shapes, precision=precision, device=DEV)
+        batch.set_persistent(persistent)
+        out.append(batch.solve(gammas, normals, prm))
+        batch.close()
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert a["status"] == b["status"] == 0 and a["iters"] == b["iters"]
+            assert abs(a["gamma_eff"] - b["gamma_eff"]) <= bar * abs(a["gamma_eff"])
+            assert abs(a["gamma_primal"] - b["gamma_primal"]) <= bar * abs(a["gamma_primal"])
+            assert abs(a["residual"] - b["residual"]) <= bar * a["mean_v_norm"]

@@ -86,3 +86,33 @@ out["one"], out["even"], out["odd"] = names(1, N + 1), names(2, N), names(2, N +
     assert _vector_kernels(got["odd"]) == []
     assert got["one"] and got["even"]
     assert _vector_kernels(got["even"]) == _vector_kernels(got["one"]) != []
+
+
+@pytest.mark.parametrize("double", [False, True])
+@pytest.mark.parametrize("persistent", [False, True])
+@pytest.mark.parametrize("variant", [None, 0, 3, 9, 13])
+def test_batch_with_an_unaligned_gamma_takes_scalar_loads(variant, persistent, double, tmp_path):
+    body = f"""
+N = 6 * 8 * 128
+es = 8 if {double} else 4
+code, h = ccmf.ccmf_batch_create([(6, 8, 128)] * 2, ccmf.CCMF_FP64 if {double} else ccmf.CCMF_FP32_MIXED)
+assert code == 0
+assert ccmf.ccmf_batch_set_persistent(h, {int(persistent)}) == 0
+n = ccmf.ccmf_batch_workspace_bytes(h)[1]
+def names(offset):
+    launches()
+    g = [buf(8 * N).value, buf(8 * N, offset).value]
+    ws = buf(n)
+    code = ccmf.ccmf_batch_solve(h, g, [[0, 0.6, 0.8]] * 2, ccmf.Params(fixed_iters=2).to_c(), ws, n, None, None)
+    assert code == 0, code
+    k = [k for _, k, _, _ in launches()]
+    # the timing runs of the tuning take every update variant over the same fields
+    code, _ = ccmf.ccmf_batch_autotune(h, g, [[0, 0.6, 0.8]] * 2, ws, n, 2, 1, None)
+    assert code == 0, code
+    return k, [k for _, k, _, _ in launches()]
+out["unaligned"], out["tuned"] = names(es)
+"""
+    got = run_fake(body, tmp_path, env={} if variant is None else {"CCMF_UPDATE_VARIANT": str(variant)})
+    assert got["unaligned"] and got["tuned"]
+    assert _vector_kernels(got["unaligned"]) == []
+    assert _vector_kernels(got["tuned"]) == []
