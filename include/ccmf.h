@@ -148,7 +148,10 @@ int ccmf_solve(ccmf_plan* plan, const void* gamma, long long gamma_stride, const
  * Copy the ADMM state of the workspace out (checkpoint): e and v ([batch][6][N]
  * each, device or host memory, may be NULL), and per solve the penalty rho and
  * the number of updates performed (host arrays [batch], may be NULL).
- * Synchronises the stream.
+ * Synchronises the stream. The state it reads is left as it is, but the call is no pure read: a state that
+ * the solver keeps in its compact form (FP32, see ccmf_tuning.update_variant) is expanded on the device, in
+ * the workspace's other copy of the state, which the next update overwrites anyway. So the workspace has
+ * to be writable, and no other call may use it meanwhile.
  */
 int ccmf_state_export(const ccmf_plan* plan, const void* workspace, void* e, void* v,
                       double* rho, int* iters, void* stream);

@@ -638,6 +638,20 @@ void tuning_store(const ccmf_plan* pl, const ccmf_tuning& t) {
 
 
 
+// Makes a device current for a call that leaves the caller's current device as it was.
+struct DeviceGuard {
+    int prev = -1, want;
+    bool ok;
+    explicit DeviceGuard(int device) : want(device) {
+        ok = cudaGetDevice(&prev) == cudaSuccess && (prev == want || cudaSetDevice(want) == cudaSuccess);
+    }
+    ~DeviceGuard() {
+        if (ok && prev != want) cudaSetDevice(prev);
+    }
+    DeviceGuard(const DeviceGuard&) = delete;
+    DeviceGuard& operator=(const DeviceGuard&) = delete;
+};
+
 bool is_device_ptr(const void* ptr) {
     if (!ptr) return false;
     cudaPointerAttributes a;
@@ -1246,6 +1260,8 @@ int ccmf_solve(ccmf_plan* plan, const void* gamma, long long gamma_stride, const
 int ccmf_state_export(const ccmf_plan* plan, const void* workspace, void* e, void* v, double* rho, int* iters,
                       void* stream) {
     if (!plan || !workspace) return CCMF_ERR_INVALID_ARG;
+    const DeviceGuard dev(plan->device);   // the expansion below is a kernel
+    if (!dev.ok) return CCMF_ERR_CUDA;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const unsigned char* ws = reinterpret_cast<const unsigned char*>(workspace);
     std::vector<SolveScalars> sc(plan->batch);

@@ -116,3 +116,38 @@ out["unaligned"], out["tuned"] = names(es)
     assert got["unaligned"] and got["tuned"]
     assert _vector_kernels(got["unaligned"]) == []
     assert _vector_kernels(got["tuned"]) == []
+
+
+def test_state_export_runs_on_the_device_of_its_plan(tmp_path):
+    """Exporting a compact FP32 state launches a kernel: on the plan's device, whichever is current, and the caller's
+    current device stays."""
+    body = _PLAN + """
+h, n = plan_for((6, 8, 16), 1, ccmf.CCMF_FP32_MIXED)
+N = 6 * 8 * 16
+ws, e, v = buf(n), buf(24 * N), buf(24 * N)
+assert ccmf.ccmf_state_import(h, ws, e, v, [0.5], [12345], None) == 0
+words = np.ctypeslib.as_array(ctypes.cast(ws, ctypes.POINTER(ctypes.c_int32)), (64,))   # the scalars of solve 0
+assert (words == 12345).sum() == 1
+imported = words.copy()
+launches()
+set_device(3)
+seen = []
+# which word holds the mark of a compact state is the library's own business: try them all
+for i in range(64):
+    for mark in (12345, 12346):
+        words[:] = imported
+        if words[i] == 12345:
+            continue
+        words[i] = mark
+        code, rho, iters = ccmf.ccmf_state_export(h, ws, e, v, 1, None)
+        assert code == 0
+        seen += [(d, k) for d, k, _, _ in launches()]
+out["seen"] = seen
+d = ctypes.c_int()
+fake.cudaGetDevice(ctypes.byref(d))
+out["current"] = d.value
+"""
+    got = run_fake(body, tmp_path)
+    assert len(got["seen"]) == 1 and "k_state_to_ev" in got["seen"][0][1]
+    assert got["seen"][0][0] == 0
+    assert got["current"] == 3
