@@ -1273,7 +1273,7 @@ int ccmf_state_export(const ccmf_plan* plan, const void* workspace, void* e, voi
     // update overwrites
     const size_t one = plan->esize * 6 * (size_t)plan->g.N;
     const size_t copy = one * plan->batch;
-    auto is_zs = [&](int s) { return plan->prec == CCMF_FP32_MIXED && sc[s].zs_iter == sc[s].iters; };
+    auto is_zs = [&](int s) { return plan->prec == CCMF_FP32_MIXED && sc[s].zs_iter == sc[s].iters + 1; };
     bool any_zs = false;
     for (int s = 0; s < plan->batch; ++s) any_zs = any_zs || is_zs(s);
     if (any_zs && (e || v)) {
@@ -1321,7 +1321,7 @@ int ccmf_state_import(const ccmf_plan* plan, void* workspace, const void* e, con
         sc[s].rho = rho[s];
         sc[s].iters = iters[s];
         sc[s].ab_iter = -1;   // stored divergences are recomputed from the imported state
-        sc[s].zs_iter = -1;   // an (e, v) state
+        sc[s].zs_iter = 0;   // an (e, v) state
     }
     if (cudaMemcpyAsync(ws + plan->off_sc, sc.data(), sizeof(SolveScalars) * plan->batch, cudaMemcpyHostToDevice,
                         st) != cudaSuccess)

@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kThreads) k_init_stats(Geom g, Ptrs<T> p, Loop
             S.rho = cfg.rho_sched ? cfg.rho_sched[(size_t)s * cfg.sched_len] : rho0;
             S.iters = 0;
             S.ab_iter = -1;
-            S.zs_iter = p.zs ? 0 : -1;
+            S.zs_iter = p.zs ? 1 : 0;
             S.rho_prev = 1.0;
         }
         S.status = status;
@@ -1406,7 +1406,7 @@ __device__ void update_finish(const Geom& g, const Ptrs<T>& p, const LoopConfig&
     const int done = kk + 1 - call_start;
     S.iters = kk + 1;
     S.ab_iter = AB ? kk + 1 : -1;   // whether the pass also wrote the divergences of the new state
-    S.zs_iter = ZS ? kk + 1 : -1;   // the format of the new state
+    S.zs_iter = ZS ? kk + 2 : 0;   // the format of the new state
     S.rho_prev = rho_d;
     bool stop = false;
     if (S.status != 0) {

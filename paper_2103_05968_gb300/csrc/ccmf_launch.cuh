@@ -663,7 +663,7 @@ __global__ void k_adj_restore(SolveScalars* sc, int batch, int k0, const double*
     sc[s].active = 1;
     sc[s].counter = 0;
     sc[s].chunk = 0;
-    sc[s].zs_iter = -1;
+    sc[s].zs_iter = 0;
 }
 
 template <typename T>
@@ -672,7 +672,6 @@ __global__ void k_adj_dummy(SolveScalars* sc, int batch) {
     if (s >= batch) return;
     SolveScalars z = {};
     z.rho = 1.0;   // w = e - v / rho with e = y, v = 0: the passes apply M to y
-    z.zs_iter = -1;
     sc[s] = z;
 }
 

@@ -11,7 +11,7 @@
 // and keeps (e, v): three more operations a component would cost it more than the bytes.
 //
 // A state that no update wrote (an imported one, or one that an update variant with the (e, v) format
-// left) has S.zs_iter != S.iters: it is read in the (e, v) format, and the first update writes (z, s).
+// left) has S.zs_iter != S.iters + 1: it is read in the (e, v) format, and the first update writes (z, s).
 //
 // Packs. The arithmetic runs on Pk<T>::V: two voxels of FP32 per register pair (the packed
 // add / mul / fma of sm_100 and later, half the issue slots), one voxel in FP64. Every product that feeds
@@ -243,7 +243,7 @@ __device__ __forceinline__ StateSrc<T> state_src(const Ptrs<T>& p, const SolveSc
 // Whether the current state of a solve is in the (z, s) format.
 template <typename T>
 __device__ __forceinline__ bool state_is_zs(const SolveScalars& S) {
-    return sizeof(T) == 4 && S.zs_iter == S.iters;
+    return sizeof(T) == 4 && S.zs_iter == S.iters + 1;
 }
 
 // (e, v, w = e - v / rho) of a pack from what the format stores: (z, s) or (e, v).

@@ -70,7 +70,8 @@ struct SolveScalars {
     int bad;             // number of invalid gamma values seen at init
     unsigned int chunk;  // next work ticket of the vector update pass (dynamic schedule)
     int ab_iter;         // update count the stored divergences a, b belong to (-1: not current)
-    int zs_iter;         // update count of a state in the (z, s) format (FP32; any other value: (e, v))
+    int zs_iter;         // update count + 1 of a state in the (z, s) format (FP32; any other value, as in cleared
+                         // memory: (e, v))
     double rho_prev;     // the penalty of the update that wrote the (z, s) state
 };
 static_assert(sizeof(SolveScalars) <= 256, "scalar slot");

@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kThreads) k_state_to_ev(Geom g, Ptrs<T> p, int
 template <typename T>
 __global__ void k_state_mark_ev(SolveScalars* sc, int batch) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < batch) sc[s].zs_iter = -1;
+    if (s < batch) sc[s].zs_iter = 0;
 }
 
 }  // namespace ccmf

@@ -151,3 +151,19 @@ out["current"] = d.value
     assert len(got["seen"]) == 1 and "k_state_to_ev" in got["seen"][0][1]
     assert got["seen"][0][0] == 0
     assert got["current"] == 3
+
+
+def test_cleared_workspace_holds_no_compact_state(tmp_path):
+    """Zeroed memory exports as it is: nothing in it reads as a compact state, whose expansion divides by the penalty."""
+    body = _PLAN + """
+h, n = plan_for((6, 8, 16), 2, ccmf.CCMF_FP32_MIXED)
+N = 6 * 8 * 16
+e, v = (np.ones(12 * N, dtype=np.float32) for _ in range(2))
+launches()
+code, rho, iters = ccmf.ccmf_state_export(h, buf(n), ctypes.c_void_p(e.ctypes.data), ctypes.c_void_p(v.ctypes.data), 2,
+                                          None)
+out["code"], out["launches"] = code, launches()
+out["values"] = [float(np.abs(e).max()), float(np.abs(v).max()), float(max(rho)), int(max(iters))]
+"""
+    got = run_fake(body, tmp_path)
+    assert got == {"code": 0, "launches": [], "values": [0.0, 0.0, 0.0, 0]}
