@@ -2295,10 +2295,10 @@ __global__ void __launch_bounds__(kThreads) k_adj_pack(Geom g, const double* __r
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
                 const double zc = zs[c * N + lin];
-                nz2 += zc * zc;
+                nz2 = fma(zc, zc, nz2);
                 zo[c * N + lin] = (float)zc;
             }
-            clip = sqrt(nz2) > gs[lin];
+            clip = Proj<double>::clips(nz2, gs[lin]);
         }
         const unsigned word = __ballot_sync(0xffffffffu, clip);
         if ((threadIdx.x & 31) == 0) bo[lin >> 5] = word;

@@ -2501,14 +2501,14 @@ __global__ void __launch_bounds__(kThreads) k_adj_pre(Geom g, const T* __restric
         for (int c = 0; c < 6; ++c) {
             zc[c] = zs[c * N + lin];
             u[c] = vs[c * N + lin] - es[c * N + lin] * irho;
-            nz2 += zc[c] * zc[c];
+            nz2 = fma(zc[c], zc[c], nz2);
         }
         const T gm = gs[lin];
         const T nz = Real<T>::sqrt_(nz2);
         // the branch of P_C: taken here, or recorded by a forward pass in higher precision
         // (one bit per voxel, [solve][ceil(N / 32)] words)
         const bool clip = clip_bits ? ((clip_bits[(size_t)s * ((N + 31) / 32) + (lin >> 5)] >> (lin & 31)) & 1u) != 0
-                                    : nz > gm;
+                                    : Proj<T>::clips(nz2, gm);
         if (clip) {
 #pragma unroll
             for (int c = 0; c < 6; ++c) zu += zc[c] * u[c];

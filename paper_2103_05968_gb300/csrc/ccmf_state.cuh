@@ -135,11 +135,15 @@ __device__ __forceinline__ bool positive_greater(double a, double b) {
     return __double_as_longlong(a) > __double_as_longlong(b);
 }
 
-// Projection helpers: scale = gamma / |z| when |z| > gamma, else 1, and norm = |x|, from squared norms. FP64
+// Projection helpers: clips = |z| > gamma, scale = gamma / |z| where it clips, else 1, and norm = |x|, from squared
+// norms. The reverse mode differentiates the branch that clips gives: it calls it on the same fma chain. FP64
 // compares squares and uses rsqrt_halley where the square lies inside float's range, the IEEE square root and
 // division elsewhere. FP32 uses the hardware reciprocal square root (relative error ~1e-7, below FP32 field noise).
 template <typename T> struct Proj;
 template <> struct Proj<double> {
+    __device__ __forceinline__ static bool clips(double nz2, double gm) {
+        return in_float_range(nz2) ? positive_greater(nz2, gm * gm) : sqrt(nz2) > gm;
+    }
     __device__ __forceinline__ static double scale(double nz2, double gm) {
         double s = 1.0;
         if (in_float_range(nz2)) {
@@ -155,8 +159,9 @@ template <> struct Proj<double> {
     }
 };
 template <> struct Proj<float> {
+    __device__ __forceinline__ static bool clips(float nz2, float gm) { return nz2 > gm * gm; }
     __device__ __forceinline__ static float scale(float nz2, float gm) {
-        return (nz2 > gm * gm) ? gm * rsqrtf(nz2) : 1.0f;
+        return clips(nz2, gm) ? gm * rsqrtf(nz2) : 1.0f;
     }
     __device__ __forceinline__ static float norm(float x2) { return x2 > 0.0f ? x2 * rsqrtf(x2) : 0.0f; }
 };
