@@ -451,6 +451,8 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     sh.smem_plane = 0;
     const size_t smem1 = ((size_t)n1 + n2 + (size_t)n1 * (n2 + 1)) * cs;
     const bool one_fits = (long long)n1 * n2 <= kPlaneMax && smem1 <= kSmemMax;
+    // line lengths of the one-warp-per-line passes
+    auto warp_len_ok = [](int n) { return n >= 128 && n <= 1024 && (n & (n - 1)) == 0; };
     int pb = r.plane_blocks;
     if (pb < 0) {
         const char* envp = getenv("CCMF_PLANE_FUSED");
@@ -461,8 +463,13 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
             pb = atoi(envc);
         else
             // FP64: one block per plane is bound by its SM's arithmetic, so the line passes win unless the planes
-            // fill the SMs twice (80^3: 41 planes take 192 us, the three line passes 86 us)
-            pb = one_fits && (!f64 || (long long)pl->n3h * batch >= 2 * sms) ? 1 : 0;
+            // fill the SMs twice (80^3: 41 planes take 192 us, the three line passes 86 us; with 304 planes and more
+            // the plane pass takes 2 to 10 % off an iteration). The in-place line passes give the plane pass's bits,
+            // so a solve is the same alone and in a batch; the warp lines do not, so where an axis has them the batch
+            // does not decide.
+            pb = one_fits && (!f64 || (!warp_len_ok(n1) && !warp_len_ok(n2) && (long long)pl->n3h * batch >= 2 * sms))
+                     ? 1
+                     : 0;
     }
     if (pb == 1) {
         if (!one_fits) return CCMF_ERR_UNSUPPORTED_SIZE;
@@ -507,7 +514,6 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     }
     if (le > 2) return CCMF_ERR_UNSUPPORTED_SIZE;
     r.line_engine = le;
-    auto warp_len_ok = [](int n) { return n >= 128 && n <= 1024 && (n & (n - 1)) == 0; };
     sh.wl_y = sh.wl_x = 0;
     sh.x_tma = 0;
     if (!sh.plane_fused && le >= 1) {

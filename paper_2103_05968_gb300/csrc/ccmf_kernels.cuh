@@ -793,7 +793,8 @@ __device__ __forceinline__ void plane_gain_stage(C* tile, int n1, int n2, int P2
         const T l2 = rsym2[c];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const T lam = rsym1[b * R + r] + l2 + l3;
+            // FP64 adds in the order of the line passes: a plan takes either by its batch, with the same bits
+            const T lam = sizeof(T) == 8 ? rsym1[b * R + r] + (l2 + l3) : rsym1[b * R + r] + l2 + l3;
             const T gk = (lam > T(0)) ? poisson_gain_div(inv_n, lam) : T(0);
             // conj: the inverse runs as conj(DIT(conj)); rounded here, not fused into the next stage's sums
             v[r] = cmake<C>(mul_rn(v[r].x, gk), mul_rn(-v[r].y, gk));
