@@ -461,6 +461,8 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
             pb = 0;
         else if (envc && atoi(envc) > 0)
             pb = atoi(envc);
+        else if (envp)
+            pb = one_fits ? 1 : 0;
         else
             // FP64: one block per plane is bound by its SM's arithmetic, so the line passes win unless the planes
             // fill the SMs twice (80^3: 41 planes take 192 us, the three line passes 86 us; with 304 planes and more

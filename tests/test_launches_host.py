@@ -167,3 +167,17 @@ out["values"] = [float(np.abs(e).max()), float(np.abs(v).max()), float(max(rho))
 """
     got = run_fake(body, tmp_path)
     assert got == {"code": 0, "launches": [], "values": [0.0, 0.0, 0.0, 0]}
+
+
+def test_plane_pass_by_environment(tmp_path):
+    """CCMF_PLANE_FUSED: 0 the line passes, another value the plane pass where a plane fits a block, unset the
+    built-in rule (in FP64 the line passes unless the planes fill the SMs twice)."""
+    body = _PLAN + """
+def info(shape, double):
+    h, _ = plan_for(shape, 1, ccmf.CCMF_FP64 if double else ccmf.CCMF_FP32_MIXED)
+    return ccmf.ccmf_plan_launch_info(h)[1]["plane_blocks"]
+out["fused"] = [info((80, 80, 80), True), info((80, 80, 80), False), info((512, 512, 16), True)]
+"""
+    assert run_fake(body, tmp_path)["fused"] == [0, 1, 0]
+    assert run_fake(body, tmp_path, env={"CCMF_PLANE_FUSED": "1"})["fused"] == [1, 1, 0]
+    assert run_fake(body, tmp_path, env={"CCMF_PLANE_FUSED": "0"})["fused"] == [0, 0, 0]
