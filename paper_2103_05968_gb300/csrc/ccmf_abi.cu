@@ -423,10 +423,7 @@ int shape_for(const ccmf_plan* pl, const ccmf_tuning& t, LaunchShape* out, ccmf_
     if (explicit_variant && sh.upd_variant != variant) return CCMF_ERR_UNSUPPORTED_SIZE;
     r.update_variant = sh.upd_variant;
     {
-        const int kind = n3 % 2 != 0 ? kUpdStrided
-                         : sh.upd_variant == 11 ? kUpdHalf2
-                         : sh.upd_variant == 12 || n3 % W != 0 ? kUpdHalf3
-                                                               : kUpdFull;
+        const int kind = update_kind(sh.upd_variant, n3 % 2 == 0, n3 % W == 0);
         const int okind = n3 % W != 0 ? kUpdStrided : kUpdFull;
         sh.upd_resident = (f64 ? update_blocks_per_sm<double>(kind, false) : update_blocks_per_sm<float>(kind, false)) * sms;
         sh.out_resident = (f64 ? update_blocks_per_sm<double>(okind, true) : update_blocks_per_sm<float>(okind, true)) * sms;
@@ -1494,12 +1491,21 @@ int ccmf_tuning_import(const char* text) {
 int ccmf_plan_launch_info(const ccmf_plan* plan, int* out, int capacity, int* count) {
     if (!plan || !count || (capacity > 0 && !out)) return CCMF_ERR_INVALID_ARG;
     const LaunchShape& sh = plan->sh;
-    const int grid_upd = is_abw_variant(sh.upd_variant) ? (int)ceil_div((long long)sh.ab.nq * sh.ab.nr * sh.ab.npass, kAbwWarps)
-                         : is_ab_variant(sh.upd_variant) ? sh.ab.nq * sh.ab.nr
-                         : (sh.upd_variant == 11 || sh.upd_variant == 12) ? sh.upd_resident / std::max(1, plan->batch)
-                         : sh.upd_variant >= 2 ? sh.grid_pipe
-                         : sh.upd_variant == 1 ? sh.grid_tma
-                                               : sh.grid_update;
+    int grid_upd = 0;
+    if (is_abw_variant(sh.upd_variant)) {
+        grid_upd = (int)ceil_div((long long)sh.ab.nq * sh.ab.nr * sh.ab.npass, kAbwWarps);
+    } else if (is_ab_variant(sh.upd_variant)) {
+        grid_upd = sh.ab.nq * sh.ab.nr;
+    } else if (!is_register_variant(sh.upd_variant)) {
+        grid_upd = sh.upd_variant >= 2 ? sh.grid_pipe : sh.grid_tma;
+    } else {
+        // of the launch of the largest branch, with gamma aligned
+        const bool f64 = plan->prec == CCMF_FP64;
+        const int W = f64 ? 2 : 4, solves = (int)ceil_div(plan->batch, std::max(1, plan->branches));
+        const int kind = update_kind(sh.upd_variant, plan->n3 % 2 == 0, plan->n3 % W == 0);
+        grid_upd = f64 ? update_grid<double>(sh, plan->g.N, solves, sh.upd_resident, kind)
+                       : update_grid<float>(sh, plan->g.N, solves, sh.upd_resident, kind);
+    }
     const int v[8] = {sh.upd_variant, sh.plane_fused, sh.plane_fused ? sh.plane_cluster : 0, sh.pairs_per_block,
                       sh.lpb_y, sh.lpb_x, grid_upd, plan->branches};
     for (int i = 0; i < 8 && i < capacity; ++i) out[i] = v[i];

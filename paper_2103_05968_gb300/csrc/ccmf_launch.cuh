@@ -235,14 +235,28 @@ int update_blocks_per_sm(int kind, bool out) {
     return a < 1 ? 1 : a;
 }
 
-// The kernel of the register update pass of a context.
+// The kernel of the register update pass, by whether gamma and N3 allow pairs and 16-byte vectors.
+inline int update_kind(int variant, bool pair, bool vec) {
+    if (!pair) return kUpdStrided;
+    if (variant == 11) return kUpdHalf2;
+    // variant 12, and every N3 = 2 mod 4 (where the plan resolves to variant 0)
+    return variant == 12 || !vec ? kUpdHalf3 : kUpdFull;
+}
+
 template <typename T>
 int update_kind(const Ctx<T>& c) {
     if (sizeof(T) == 4 && !c.use_zs) return kUpdStridedEv;
-    if (!c.pair_update) return kUpdStrided;
-    if (c.sh.upd_variant == 11) return kUpdHalf2;
-    // variant 12, and every N3 = 2 mod 4 (where the plan resolves to variant 0)
-    return c.sh.upd_variant == 12 || !c.vec_update ? kUpdHalf3 : kUpdFull;
+    return update_kind(c.sh.upd_variant, c.pair_update, c.vec_update);
+}
+
+// Blocks per solve of a register update pass over `solves` solves: the resident blocks, shared by the solves, so that
+// every solve's chunks run at once on all SMs, and no more than a solve has chunks.
+template <typename T>
+int update_grid(const LaunchShape& sh, long long n_voxels, int solves, int resident, int kind) {
+    const long long chunks = vec_update_chunks<T>(n_voxels, update_voxels<T>(kind));
+    long long b = resident > 0 ? resident / solves : sh.grid_update;
+    b = b < chunks ? b : chunks;
+    return (int)(b < 1 ? 1 : b);
 }
 
 #define CCMF_DISPATCH_ABW(var, ...)                                                      \
@@ -458,13 +472,9 @@ void launch_passes(const Ctx<T>& c, const Ptrs<T>& p, cudaStream_t st, F&& betwe
     if (sh.grid_x > 0 && sh.grid_x < twx) twx = sh.grid_x;
     dim3 gwy((unsigned)twy, (unsigned)g.batch);
     dim3 gwx((unsigned)twx, (unsigned)g.batch);
-    // the register update pass takes its chunks from a ticket counter: the resident blocks, shared
-    // by the solves of this launch, so that every solve's chunks run at once on all SMs
+    // the register update pass takes its chunks from a ticket counter
     auto grid_upd = [&](int resident, int kind) {
-        const long long chunks = vec_update_chunks<T>(g.N, update_voxels<T>(kind));
-        long long b = resident > 0 ? resident / g.batch : sh.grid_update;
-        b = b < chunks ? b : chunks;
-        return dim3((unsigned)(b < 1 ? 1 : b), (unsigned)g.batch);
+        return dim3((unsigned)update_grid<T>(sh, g.N, g.batch, resident, kind), (unsigned)g.batch);
     };
     const T inv_n = (T)(poisson_scale<T>() / (double)g.N);
     const dim3 gwz((unsigned)ceil_div((long long)g.n1 * g.n2, 2 * (kThreads / 32)), (unsigned)g.batch);

@@ -181,3 +181,23 @@ out["fused"] = [info((80, 80, 80), True), info((80, 80, 80), False), info((512, 
     assert run_fake(body, tmp_path)["fused"] == [0, 1, 0]
     assert run_fake(body, tmp_path, env={"CCMF_PLANE_FUSED": "1"})["fused"] == [1, 1, 0]
     assert run_fake(body, tmp_path, env={"CCMF_PLANE_FUSED": "0"})["fused"] == [0, 0, 0]
+
+
+@pytest.mark.parametrize("double", [False, True])
+@pytest.mark.parametrize("variant", [0, 11, 12])
+@pytest.mark.parametrize("shape,batch", [((6, 8, 16), 1), ((64, 64, 64), 3), ((128, 128, 128), 1), ((50, 48, 32), 7)])
+def test_launch_info_names_the_grid_of_the_update_pass(shape, batch, variant, double, tmp_path):
+    body = _PLAN + f"""
+shape, batch = {shape}, {batch}
+h, n = plan_for(shape, batch, ccmf.CCMF_FP64 if {double} else ccmf.CCMF_FP32_MIXED, update_variant={variant})
+N = shape[0] * shape[1] * shape[2]
+launches()
+code = ccmf.ccmf_solve(h, buf(8 * N), 0, [[0, 0.6, 0.8]] * batch, ccmf.Params(fixed_iters=2).to_c(), buf(n), n, None, None,
+                       None, None)
+assert code == 0
+out["grids"] = [g for _, k, g, _ in launches() if "k_update" in k][:-1]    # the last is the final evaluation
+out["said"] = ccmf.ccmf_plan_launch_info(h)[1]["update_blocks"]
+"""
+    got = run_fake(body, tmp_path)
+    # the smallest grid is that of the branch with the most solves
+    assert min(got["grids"]) == got["said"]
