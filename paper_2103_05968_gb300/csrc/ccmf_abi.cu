@@ -1637,7 +1637,9 @@ int batch_persist_capture(ccmf_batch* bt, const std::vector<Ctx<T>>& ctx, unsign
         G.tiles[4] = G.tiles[0];
         G.tiles[5] = (int)G.nchunks;
         // bytes one tile of each pass moves (FP32 fields; FP64 doubles them): items of about
-        // 256 KB keep the per-item cost (ticket, barriers, release) small against the tile work
+        // 256 KB keep the per-item cost (ticket, barriers, release) small against the tile work.
+        // Pass 0 counts the 52 B/voxel of an (e, v) state; on (z, s) it moves 32, so its FP32 items
+        // are about 160 KB
         const double es = (double)sizeof(T) / 4.0;
         const double tile_bytes[kPersistPasses] = {2.0 * P * pl->n3 * 52.0 * es, (double)L * pl->n2 * 16.0 * es,
                                                    (double)L * pl->n1 * 16.0 * es, (double)L * pl->n2 * 16.0 * es,

@@ -1051,15 +1051,13 @@ __global__ void __launch_bounds__(kThreads, wz_min_blocks<T, N>())
             } else if (valid) {
                 const int kp = (k0 + W == N) ? 0 : k0 + W;   // first voxel after the group
                 const int km = (k0 == 0) ? N - 1 : k0 - 1;   // last voxel before the group
-                if constexpr (AB) {
-                } else if constexpr (sizeof(T) == 4) {
-                    if (zs)
-                        div_group<T, true>(f, rn, k0, kp, km, d);
-                    else
-                        div_group<T, false>(f, rn, k0, kp, km, d);
-                } else {
-                    div_group<T, false>(f, rn, k0, kp, km, d);
-                }
+                auto div = [&](auto fmt) {
+                    if constexpr (!AB) div_group<T, decltype(fmt)::value>(f, rn, k0, kp, km, d);
+                };
+                if (sizeof(T) == 4 && zs)
+                    div(BoolC<sizeof(T) == 4>{});
+                else
+                    div(BoolC<false>{});
             }
             // line 2w + q is the real (q = 0) or imaginary (q = 1) part of packed line w
 #pragma unroll

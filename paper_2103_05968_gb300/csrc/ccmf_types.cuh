@@ -33,6 +33,8 @@ constexpr int kThreads = 256;
 // above it they stay whole (256^3: 211 us with 16 groups, 237 us with five rounds of 15, whose ends cut rows).
 // FP64, where a group's arithmetic is long: halved from 16 until there are kVecMinChunks (128^3 update 735 us with
 // 96, 741 with 400, 700 with 1300).
+// 456 is the residency of update variant 12, the FP32 default. The final evaluation (one block per SM), variant 0 (one)
+// and variant 11 (two) keep the same chunks, one partial slot each, and take them in more rounds.
 // The rule depends on the grid and the precision alone, so a solve sums in the same order alone and in a batch.
 constexpr int kVecChunkGroups = 16;
 template <typename T>
