@@ -810,7 +810,7 @@ def run_gpu(args, world, rank, local):
             "solver_fft_passes_ms": sum(kt[k][0] / kt[k][1] for k in fft_cls),
             "solver_passes": fft_cls,
             "note": "cuFFT: torch.fft.rfftn + irfftn of B real grids; solver: its forward and inverse FFT "
-                    "passes per iteration (the first also reads e, v and computes the divergence; the plane "
+                    "passes per iteration (the first also reads the state and computes the divergence; the plane "
                     "pass also applies the Poisson symbol), sequential event timing"}
 
     # FP32-mixed vs plain FP64 time to relative gamma_eff error 1e-5 (default workload, rank 0)

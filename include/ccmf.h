@@ -192,8 +192,8 @@ int ccmf_kernel_times(const ccmf_plan* plan, double* ms, long long* launches, co
  * plane pass fused (0 / 1),
  * blocks sharing one (x, y) plane (1 = one block, 2..16 = a thread-block cluster),
  * z-pass line pairs per block, y-pass lines per block, x-pass lines per block,
- * update-pass blocks per solve, graph branches}. Writes min(capacity, 8) entries and
- * returns 8 in *count.
+ * update-pass blocks per solve (in the launch of the largest branch), graph branches}.
+ * Writes min(capacity, 8) entries and returns 8 in *count.
  */
 int ccmf_plan_launch_info(const ccmf_plan* plan, int* out, int capacity, int* count);
 

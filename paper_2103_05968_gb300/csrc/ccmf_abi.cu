@@ -70,12 +70,12 @@ constexpr int kMaxN = 1024;
 constexpr size_t kSmemBudget = 96 * 1024;
 constexpr size_t kSmemMax = 200 * 1024;   // dynamic shared memory of one block, at most
 constexpr int kMaxTimedIters = 2048;
-// update-pass variant per precision, from measurements on GB300: register vectors in
-// ticket-ordered chunks. FP32 waits for memory: half the voxels per thread and three blocks per SM
-// (variant 12, 80 registers, no spills) take 1.58 ms per 512^3 pass against 1.79 ms with two blocks (variant 11) and
-// 1.86 ms with one block of 16-byte vectors (variant 0); 0.236 / 0.266 / 0.274 ms at 256^3. FP64 is ALU-bound and wants
-// its voxels spread over the SMs: one voxel per thread (variant 11) takes 27 us per 32^3 pass against 37 us with
-// 16-byte vectors, 0.631 against 0.649 ms at 128^3.
+// update-pass variant per precision, from measurements on GB300: register vectors in ticket-ordered chunks. FP32 waits
+// for memory: half the voxels per thread and three blocks per SM (variant 12, 80 registers, no spills) take 1.53 ms per
+// 512^3 pass against 1.72 ms with two blocks (variant 11) and 1.81 ms with one block of 16-byte vectors (variant 0);
+// 0.211 / 0.242 / 0.247 ms at 256^3, 0.093 / 0.105 / 0.111 ms for three 128^3 solves. FP64 is ALU-bound and wants its
+// voxels spread over the SMs: one voxel per thread (variant 11) takes 27 us per 32^3 pass against 36 us with 16-byte
+// vectors, 0.594 against 0.617 ms at 128^3.
 constexpr int kDefaultUpdateVariantF32 = 12;
 constexpr int kDefaultUpdateVariantF64 = 11;
 // the captured loop runs the solves of a batch as up to this many independent graph

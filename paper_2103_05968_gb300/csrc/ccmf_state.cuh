@@ -7,7 +7,7 @@
 // reader forms v = s z, e = (z - v) / rho_prev with the very operations that the update uses for its
 // own sums. The update is bound by HBM: it moves 36 + 28 B/voxel instead of 56 + 48, and the
 // divergence pass 28 + 4 instead of 48 + 4. Measured on GB300, 512^3: update 2.37 -> 1.53 ms,
-// divergence pass 1.09 -> 0.87 ms. FP64 is bound by its arithmetic (1/64 of the FP32 rate)
+// divergence pass 1.09 -> 0.89 ms. FP64 is bound by its arithmetic (1/64 of the FP32 rate)
 // and keeps (e, v): three more operations a component would cost it more than the bytes.
 //
 // A state that no update wrote (an imported one, or one that an update variant with the (e, v) format
