@@ -1226,7 +1226,7 @@ template <typename T>
 struct StepConsts {
     T rho, irho, h, alpha, beta;
     T xi[3];
-    T hxi[3];   // xi_bar / sqrt2
+    T hxi[3];   // xi_bar / sqrt2, sqrt(1/2) rounded down
 };
 
 // Per-voxel work of the update pass. Inputs: the voxel's own state (ec, vc),
@@ -1438,13 +1438,16 @@ __device__ __forceinline__ StepConsts<T> step_consts(const SolveScalars& S, cons
     K.h = T(0.70710678118654752440084436210485);
     K.alpha = (T)(2.0 * (1.0 - cfg.delta));
     K.beta = (T)(1.0 - 2.0 * cfg.delta);
-    const double hd = 0.70710678118654752440084436210485;
+    // The two doubles next to sqrt(1/2) are equally far from it. The default start has |z| = rho0 = min gamma up to
+    // rounding on the weakest phase (e^0 = A xi_bar, k_init_state, with the upper one): with the lower one here the first
+    // z lies just below gamma and e' = 0 stays exact, as the LTD rule needs it. FP64 only (fold_h).
+    const double hd_down = 0.70710678118654746171500846685376;
     K.xi[0] = (T)S.xi[0];
     K.xi[1] = (T)S.xi[1];
     K.xi[2] = (T)S.xi[2];
-    K.hxi[0] = (T)(S.xi[0] * hd);
-    K.hxi[1] = (T)(S.xi[1] * hd);
-    K.hxi[2] = (T)(S.xi[2] * hd);
+    K.hxi[0] = (T)(S.xi[0] * hd_down);
+    K.hxi[1] = (T)(S.xi[1] * hd_down);
+    K.hxi[2] = (T)(S.xi[2] * hd_down);
     return K;
 }
 

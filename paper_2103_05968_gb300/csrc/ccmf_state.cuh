@@ -126,28 +126,32 @@ __device__ __forceinline__ double rsqrt_halley(double x) {
     const double e = fma(-x, y * y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
-// 2^-100 <= x < 2^100, and a > b for values that are not negative, on the bits (comparisons of doubles occupy the FP64
-// unit too; a NaN compares as larger than anything and passes through the projection as a NaN either way).
+// 2^-100 <= x < 2^100, on the bits (a comparison of doubles occupies the FP64 unit too).
 __device__ __forceinline__ bool in_float_range(double x) {
     return (unsigned)(__double2hiint(x) - (923 << 20)) < (200u << 20);
 }
-__device__ __forceinline__ bool positive_greater(double a, double b) {
-    return __double_as_longlong(a) > __double_as_longlong(b);
+// sqrt(x) > g for the correctly rounded square root, without taking it: the root rounds up past g where it exceeds the
+// middle of g and its successor g', that is where x > g g' (what (g + g')^2 / 4 adds to that is too little for a double
+// x to lie between). The fma rounds g g' - x once, so its sign is exact. x > g^2 would be one ulp of x too sharp: before
+// the first update |z| = rho0 = min gamma on a whole phase, and a rounding error there would pass for a clipped voxel.
+__device__ __forceinline__ bool root_exceeds(double x, double g) {
+    const double next = __longlong_as_double(__double_as_longlong(g) + 1);
+    return __double2hiint(fma(g, next, -x)) < 0;
 }
 
 // Projection helpers: clips = |z| > gamma, scale = gamma / |z| where it clips, else 1, and norm = |x|, from squared
 // norms. The reverse mode differentiates the branch that clips gives: it calls it on the same fma chain. FP64
-// compares squares and uses rsqrt_halley where the square lies inside float's range, the IEEE square root and
-// division elsewhere. FP32 uses the hardware reciprocal square root (relative error ~1e-7, below FP32 field noise).
+// decides as the IEEE square root would and uses rsqrt_halley where the square lies inside float's range, the IEEE
+// square root and division elsewhere. FP32 compares squares and uses the hardware reciprocal square root (relative error ~1e-7, below FP32 field noise).
 template <typename T> struct Proj;
 template <> struct Proj<double> {
     __device__ __forceinline__ static bool clips(double nz2, double gm) {
-        return in_float_range(nz2) ? positive_greater(nz2, gm * gm) : sqrt(nz2) > gm;
+        return in_float_range(nz2) ? root_exceeds(nz2, gm) : sqrt(nz2) > gm;
     }
     __device__ __forceinline__ static double scale(double nz2, double gm) {
         double s = 1.0;
         if (in_float_range(nz2)) {
-            if (positive_greater(nz2, gm * gm)) s = gm * rsqrt_halley(nz2);
+            if (root_exceeds(nz2, gm)) s = gm * rsqrt_halley(nz2);
         } else {
             const double nz = sqrt(nz2);
             if (nz > gm) s = gm / nz;
